@@ -198,8 +198,8 @@ def _one_problem_workloads():
                              "binary": "k_binary_c + k_binary_small_c (and/or/U level kernels, 512-byte CMs)"}),
         "large": dict(make=lambda W, lab, seed: W.large_problem(seed, lab), cache=LARGE_CACHE_BYTES, max_size=15,
                       op_mask=0x7F, dtype="u64", desc=LARGE_WORKLOAD, steps=3, cpu_levels=(4, 5), fill=True,
-                      kernels={"unary": "k_unary_d (not/X/F/G level kernel, 16 KiB CMs)",
-                               "binary": "k_binary_d (and/or/U level kernel, 16 KiB CMs)"}),
+                      kernels={"unary": "k_group (not/X/F/G level kernel, 16 KiB CMs)",
+                               "binary": "k_group (and/or/U level kernel, 16 KiB CMs)"}),
         "e3": dict(make=lambda W, lab, seed: _paper_example(W), cache=16 << 30, max_size=16,
                    op_mask=0x1B | 0x40, dtype="u32", desc=E3_WORKLOAD, steps=5, cpu_levels=(12, 14),
                    kernels={"unary": "k_unary_a (not/X/F/G level kernel, 64-byte CMs)",

@@ -37,7 +37,7 @@ template <> struct WordInfo<uint64_t> { static constexpr int kMaxSteps = 6; };
 // The enumeration kernels use these forms (w_op):
 //   not : ~a & lenmask
 //   X   : a << 1                        (position t takes position t + 1)
-//   F   : -(a & -a)                     (every bit from the lowest set bit up:
+//   F   : a | -a                        (every bit from the lowest set bit up:
 //                                        "holds at t or at some later position")
 //   G   : not F not, masked to the trace length
 //   U   : B | (A & ((A|B) + B  ^  (A & ~B)))   with A = phi, B = psi.
@@ -53,7 +53,7 @@ template <> struct WordInfo<uint64_t> { static constexpr int kMaxSteps = 6; };
 // ---------------------------------------------------------------------------
 template <typename W>
 __device__ __forceinline__ W w_future(W a) {
-  return W(0) - (a & (W(0) - a));
+  return a | (W(0) - a);
 }
 
 template <typename W>
@@ -303,6 +303,18 @@ __device__ __forceinline__ uint32_t spec_bad(uint4 c, uint4 lab, uint4 care) {
          ((c.w ^ lab.w) & care.w);
 }
 
+// The same with the words' top bits left in place: bit 31 of the result is set
+// when a position-0 bit of c differs from its trace's label (the other bits
+// mean nothing; padding words are 0 with label 0). One three-input logic
+// operation a word.
+template <typename W> __device__ __forceinline__ uint32_t label_miss(uint4 c, uint4 lab);
+template <> __device__ __forceinline__ uint32_t label_miss<uint32_t>(uint4 c, uint4 lab) {
+  return (c.x ^ lab.x) | (c.y ^ lab.y) | (c.z ^ lab.z) | (c.w ^ lab.w);
+}
+template <> __device__ __forceinline__ uint32_t label_miss<uint64_t>(uint4 c, uint4 lab) {
+  return (c.y ^ lab.y) | (c.w ^ lab.w);
+}
+
 __device__ __forceinline__ uint32_t v_ne(uint4 a, uint4 b) {
   return (a.x ^ b.x) | (a.y ^ b.y) | (a.z ^ b.z) | (a.w ^ b.w);
 }
@@ -391,6 +403,10 @@ __device__ __forceinline__ const uint4* row_ptr(const CacheView& cv, uint32_t id
 // anyway.
 __device__ __forceinline__ uint2 split_pair(const Split& S, unsigned long long local, bool large_outer) {
   if (!S.tri) {
+    if ((local >> 32) == 0ull) {  // the usual case: a 32-bit division
+      const uint32_t l = uint32_t(local), n = large_outer ? S.left_n : S.right_n, q = l / n;
+      return large_outer ? make_uint2(l - q * n, q) : make_uint2(q, l - q * n);
+    }
     if (large_outer) {
       const uint32_t ib = uint32_t(local / S.left_n);
       return make_uint2(uint32_t(local - (unsigned long long)ib * S.left_n), ib);
@@ -597,47 +613,6 @@ __device__ __forceinline__ void cp_async16(uint4* smem, const uint4* gmem) {
 
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
-// Bulk copies of whole rows into shared memory (the TMA unit's non-tensor
-// form), completed on a per-warp mbarrier: lane 0 arms the barrier with the
-// bytes to expect and issues the copies; every lane then waits on the
-// barrier's phase. Addresses are 16-byte aligned and sizes multiples of 16.
-__device__ __forceinline__ unsigned smem_u32(const void* p) {
-  return static_cast<unsigned>(__cvta_generic_to_shared(p));
-}
-__device__ __forceinline__ void mbar_init(unsigned long long* bar, unsigned count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
-  asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-}
-__device__ __forceinline__ void mbar_arrive_expect_tx(unsigned long long* bar, unsigned bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ bool mbar_try_wait(unsigned long long* bar, unsigned parity) {
-  unsigned ok;
-  asm volatile(
-      "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
-      : "=r"(ok)
-      : "r"(smem_u32(bar)), "r"(parity)
-      : "memory");
-  return ok != 0u;
-}
-__device__ __forceinline__ void bulk_load(void* dst, const void* src, unsigned bytes, unsigned long long* bar) {
-  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                   smem_u32(dst)),
-               "l"(src), "r"(bytes), "r"(smem_u32(bar))
-               : "memory");
-}
-// Orders this thread's earlier shared-memory accesses (and, after a warp
-// barrier, its warp's) before later accesses of the async proxy (bulk copies).
-__device__ __forceinline__ void fence_proxy_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
-
-// Waits for phase `parity` of the barrier, at most `limit` polls per lane;
-// warp-uniform result (false: some lane gave up).
-__device__ __forceinline__ bool mbar_wait_bounded(unsigned long long* bar, unsigned parity, unsigned limit) {
-  bool done = false;
-  for (unsigned i = 0; i < limit && !done; ++i) done = mbar_try_wait(bar, parity);
-  return __all_sync(0xFFFFFFFFu, done);
-}
-
 __device__ __forceinline__ void fence_acq_rel_gpu() { asm volatile("fence.acq_rel.gpu;" ::: "memory"); }
 
 __device__ __forceinline__ void st_relaxed(unsigned long long* p, unsigned long long v) {
@@ -778,14 +753,14 @@ struct PathC {
   using Ids = WarpDedup::Ids;
 
   struct Consts {
-    uint4 mul;     // hash multipliers of this lane's 32-bit words
-    uint32_t lab;  // bit j: 1 iff word j of this lane's vector belongs to a positive trace
+    uint4 mul;  // hash multipliers of this lane's 32-bit words
+    uint4 lab;  // top bit of a word: 1 iff it belongs to a positive trace
   };
 
   __device__ static void load_consts(const CacheView& cv, Consts& k) {
     const int lane = threadIdx.x & 31;
     k.mul = cv.hmul[lane];
-    k.lab = bit0s<W>(cv.label[lane]);
+    k.lab = cv.label[lane];
   }
 
   // The first (at most) kGroup set bits of m.
@@ -827,7 +802,7 @@ struct PathC {
         const uint32_t hi = __reduce_add_sync(kFull, uint32_t(acc >> 32));
         my_lo = lane == q ? lo : my_lo;
         my_hi = lane == q ? hi : my_hi;
-        bad |= ((bit0s<W>(c4[o]) ^ k.lab) != 0u ? 1u : 0u) << q;
+        bad |= (label_miss<W>(c4[o], k.lab) >> 31) << q;
       }
     }
     // Separation (section "Synthesising ... from examples"): the position-0 bit
@@ -1275,13 +1250,14 @@ __global__ void __launch_bounds__(256, 3) k_desc_c(CacheView cv, const unsigned 
 }
 
 // ===========================================================================
-// Path D (CMs above 512 bytes, e.g. 2048 traces of 64-bit words = 16 KiB): the
-// hash-first scheme of path C with rv = vecs / 32 vectors per lane, walked in
-// loops, VPT vectors at a time (their operand loads in flight together).
-// Operand rows are read through L1/L2 whenever a candidate is (re)computed;
-// compares read the stored row directly.
+// Path D of the batch kernels (CMs above 128 bytes, several words per trace
+// among them; one problem's own levels above 512 bytes take the group kernels,
+// lsyn_group.cuh): the hash-first scheme of path C with rv = vecs / 32 vectors
+// per lane, walked in loops, VPT vectors at a time (their operand loads in
+// flight together). Operand rows are read through L1/L2 whenever a candidate is
+// (re)computed; compares read the stored row directly.
 // ===========================================================================
-template <typename W, int VPT = 1, int CU = 1>
+template <typename W, int VPT = 1>
 struct PathD {
   using Pending = WarpDedup::Pending;
   using Ids = WarpDedup::Ids;
@@ -1396,36 +1372,13 @@ struct PathD {
 #pragma unroll
         for (int o = 0; o < 4; ++o) src[o] = row_ptr(cv, __shfl_sync(kFull, cmp_id, 4 * g + o));  // published rows, read past L1
         uint32_t ne[4] = {0u, 0u, 0u, 0u};
-        if constexpr (CU == 1) {
-          for (unsigned r = 0; r < rv; ++r) {
-            const unsigned v = lane + 32u * r;
-            uint4 c[4];
-            gen.compute4(4 * g, v, c, sub);
+        for (unsigned r = 0; r < rv; ++r) {
+          const unsigned v = lane + 32u * r;
+          uint4 c[4];
+          gen.compute4(4 * g, v, c, sub);
 #pragma unroll
-            for (int o = 0; o < 4; ++o)
-              if ((sub >> o) & 1u) ne[o] |= v_ne(__ldcg(src[o] + v), c[o]);
-          }
-        } else {
-        // CU vectors per lane of each stored row read together (their loads in
-        // flight at once), then compared
-        for (unsigned r = 0; r < rv; r += CU) {
-          uint4 st[CU][4];
-#pragma unroll
-          for (int u = 0; u < CU; ++u)
-#pragma unroll
-            for (int o = 0; o < 4; ++o)
-              st[u][o] = ((sub >> o) & 1u) && r + u < rv ? __ldcg(src[o] + lane + 32u * (r + u))
-                                                          : make_uint4(0u, 0u, 0u, 0u);
-#pragma unroll
-          for (int u = 0; u < CU; ++u) {
-            if (r + u >= rv) break;
-            uint4 c[4];
-            gen.compute4(4 * g, lane + 32u * (r + u), c, sub);
-#pragma unroll
-            for (int o = 0; o < 4; ++o)
-              if ((sub >> o) & 1u) ne[o] |= v_ne(st[u][o], c[o]);
-          }
-        }
+          for (int o = 0; o < 4; ++o)
+            if ((sub >> o) & 1u) ne[o] |= v_ne(__ldcg(src[o] + v), c[o]);
         }
 #pragma unroll
         for (int o = 0; o < 4; ++o)
@@ -1585,223 +1538,6 @@ struct ListGenD {
   }
   __device__ uint64_t desc(int q) const { return d[q]; }
 };
-
-// Rows of level k-1 per warp batch of k_unary_d (4 operators each). A batch
-// reads its rows once to hash them and again to compare or write its
-// candidates; one 16 KiB row per warp keeps the rows of all resident warps
-// in L2 between the passes (8 rows per warp did not fit, and the second reads
-// went to DRAM), and a batch's round trips stay short beside its streaming.
-constexpr int kRowsD = 1;
-// Vectors per lane computed together in the hash pass of path D: of k_unary_d
-// (one row read, four loads in flight per lane), and of k_binary_d and
-// k_desc_d. Measured at 16 KiB CMs: 4 against 1, 2 or 8 for the unary
-// kernel, 2 against 1 or 4 for the binary one.
-constexpr int kVptUnaryD = 4;
-constexpr int kVptD = 2;
-
-template <typename W>
-__global__ void __launch_bounds__(256) k_unary_d(CacheView cv, uint32_t first, uint32_t count, uint32_t ops) {
-  using P = PathD<W, kVptUnaryD>;
-  constexpr int ROWS = kRowsD;
-  const int lane = threadIdx.x & 31;
-  RowGenD<W> gen;
-  gen.cv = &cv;
-  uint32_t en_ops = 0;
-#pragma unroll
-  for (int q = 0; q < 4 * ROWS; ++q) en_ops |= ((ops >> (q & 3)) & 1u) << q;
-  const uint32_t warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const uint32_t nwarps = (gridDim.x * blockDim.x) >> 5;
-  unsigned long long built = 0;
-  typename P::Pending pend;
-  typename P::Ids idr;
-  for (uint32_t base = warp * ROWS; base < count; base += nwarps * ROWS) {
-    if (__any_sync(kFull, stop_requested(cv))) break;
-    const uint32_t nrows = min(uint32_t(ROWS), count - base);
-    gen.id0 = first + base;
-    const uint32_t en = en_ops & (nrows >= 8u ? 0xFFFFFFFFu : ((1u << (4 * nrows)) - 1u));
-    P::template batch<false>(cv, gen, int(4 * nrows), en, pend, idr);
-    built += __popc(en);
-  }
-  WarpDedup::flush(pend);
-  WarpDedup::retire(cv, idr);
-  if (lane == 0 && built) atomicAdd(&cv.ctr->built_k[cv.kind], built);
-}
-
-// Staged form of k_unary_d for one-plane CMs of 8-16 KiB. Each warp copies
-// its operand row into shared memory with one bulk copy (the TMA unit moves the
-// whole row while the warp waits on an mbarrier) and every pass of the batch
-// (hash and specification check, in-batch twins, compares, writes) computes
-// the four operators from that copy: the row is read from HBM once, where
-// k_unary_d reads it again after its probes and, with 16 KiB rows, finds it
-// evicted from L2 about a quarter of the time. Shared memory bounds the block
-// to as many warps as rows of M bytes fit its shared memory: 14 with 16 KiB
-// rows.
-constexpr unsigned kStagedMinBytes = 8192, kStagedMaxBytes = 16384;
-constexpr int kStagedMaxWarps = 16;
-constexpr unsigned kBulkChunk = 4096;        // bytes per bulk copy instruction
-constexpr unsigned kRowWaitPolls = 1u << 22; // polls of the row's barrier before the warp gives up
-// Vectors per lane of each stored row that the compare pass of k_unary_ds
-// loads together: with few warps per SM, a compare read one vector at a time
-// was a chain of 32 round trips per 16 KiB row.
-constexpr int kCmpVecsDS = 4;
-
-template <typename W>
-struct RowGenDS {
-  const CacheView* cv;
-  const uint4* row;  // shared memory: the operand row
-  uint32_t id0;
-  __device__ uint4 compute(int q, unsigned v) const {
-    const uint4 x = row[v];
-    return v_op<W>(unary_code(q & 3), x, x, __ldg(cv->lenmask + v), 0);
-  }
-  __device__ void compute4(int /*q0*/, unsigned v, uint4 (&c)[4], uint32_t /*sub*/ = 0xFu) const {
-    const uint4 x = row[v], lm = __ldg(cv->lenmask + v);
-#pragma unroll
-    for (int o = 0; o < 4; ++o) c[o] = v_op<W>(unary_code(o), x, x, lm, 0);
-  }
-  __device__ uint64_t desc(int q) const { return pack_desc(unary_code(q & 3), id0, 0); }
-};
-
-template <typename W>
-__global__ void __launch_bounds__(32 * kStagedMaxWarps) k_unary_ds(CacheView cv, uint32_t first, uint32_t count,
-                                                                   uint32_t ops) {
-  using P = PathD<W, kVptUnaryD, kCmpVecsDS>;
-  extern __shared__ __align__(128) uint4 smem_rows[];
-  __shared__ unsigned long long s_bar[kStagedMaxWarps];
-  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-  const unsigned row_bytes = cv.vecs * 16u;
-  uint4* row = smem_rows + size_t(wib) * cv.vecs;
-  unsigned long long* bar = s_bar + wib;
-  if (lane == 0) mbar_init(bar, 1u);
-  __syncwarp();
-  RowGenDS<W> gen;
-  gen.cv = &cv;
-  gen.row = row;
-  const uint32_t en = ops & 0xFu;  // the four operators of the row, as enabled
-  const uint32_t warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const uint32_t nwarps = (gridDim.x * blockDim.x) >> 5;
-  unsigned long long built = 0;
-  typename P::Pending pend;
-  typename P::Ids idr;
-  unsigned parity = 0;
-  for (uint32_t base = warp; base < count; base += nwarps) {
-    if (__any_sync(kFull, stop_requested(cv))) break;
-    // every lane's reads of the previous row are done before the copy overwrites it
-    __syncwarp();
-    if (lane == 0) {
-      fence_proxy_async_smem();
-      mbar_arrive_expect_tx(bar, row_bytes);
-      const char* src = reinterpret_cast<const char*>(row_ptr(cv, first + base));
-      char* dst = reinterpret_cast<char*>(row);
-      for (unsigned off = 0; off < row_bytes; off += kBulkChunk)
-        bulk_load(dst + off, src + off, min(kBulkChunk, row_bytes - off), bar);
-    }
-    if (!mbar_wait_bounded(bar, parity, kRowWaitPolls)) {
-      // cannot happen while the copy engine works: record it, give the copy a
-      // second bounded wait (it writes this block's shared memory) and stop
-      if (lane == 0) atomicExch(&cv.ctr->error, 6u);
-      mbar_wait_bounded(bar, parity, kRowWaitPolls);
-      break;
-    }
-    parity ^= 1u;
-    gen.id0 = first + base;
-    P::template batch<false>(cv, gen, 4, en, pend, idr);
-    built += __popc(en);
-  }
-  WarpDedup::flush(pend);
-  WarpDedup::retire(cv, idr);
-  if (lane == 0 && built) atomicAdd(&cv.ctr->built_k[cv.kind], built);
-}
-
-// Pairs of every split in one flat index space (as path A), kPairsD per warp
-// batch (4 measured faster than 8, 2 or 1 at 16 KiB CMs).
-constexpr int kPairsD = 4;
-
-template <typename W>
-__global__ void __launch_bounds__(256) k_binary_d(CacheView cv, BinaryPlan plan) {
-  using P = PathD<W, kVptD>;
-  constexpr int PAIRS = kPairsD;
-  __shared__ uint2 s_pairs[8][PAIRS];
-  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-  PairGenD<W> gen;
-  gen.cv = &cv;
-  gen.pairs = s_pairs[wib];
-  const unsigned long long warp = (blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x) >> 5;
-  const unsigned long long nwarps = ((unsigned long long)gridDim.x * blockDim.x) >> 5;
-  unsigned long long built = 0;
-  typename P::Pending pend;
-  typename P::Ids idr;
-  for (unsigned long long g0 = warp * PAIRS; g0 < plan.total_pairs; g0 += nwarps * PAIRS) {
-    if (__any_sync(kFull, stop_requested(cv))) break;
-    // lane p < PAIRS maps pair g0 + p to its operands
-    uint32_t ok = 0;
-    if (lane < PAIRS) {
-      const unsigned long long pidx = g0 + lane;
-      bool valid = pidx < plan.total_pairs;
-      uint2 pr = make_uint2(0, 0);
-      if (valid) {
-        int sp = 0;
-        while (sp + 1 < plan.n_splits && plan.s[sp + 1].pairs_begin <= pidx) ++sp;
-        const Split& S = plan.s[sp];
-        const uint2 ab = split_pair(S, pidx - S.pairs_begin, true);
-        pr = make_uint2(S.left_start + ab.x, S.right_start + ab.y);
-      }
-      s_pairs[wib][lane] = pr;
-      ok = valid ? 1u : 0u;
-    }
-    const uint32_t pv = __ballot_sync(kFull, ok != 0u) & ((1u << PAIRS) - 1u);
-    __syncwarp();
-    uint32_t en = 0;
-#pragma unroll
-    for (int q = 0; q < 4 * PAIRS; ++q) en |= (((pv >> (q >> 2)) & 1u) & ((plan.ops >> (q & 3)) & 1u)) << q;
-    if (en) {
-      P::template batch<true>(cv, gen, 4 * PAIRS, en, pend, idr);
-      built += __popc(en);
-    }
-    __syncwarp();
-  }
-  WarpDedup::flush(pend);
-  WarpDedup::retire(cv, idr);
-  if (lane == 0 && built) atomicAdd(&cv.ctr->built_k[cv.kind], built);
-}
-
-// Descriptors per warp batch of k_desc_d: one group of four. A path-D batch
-// walks its groups one after another, each a chain of passes over the
-// candidates' vectors, so a short deferred list (the usual case) spreads over
-// many warps instead of queueing in a few.
-constexpr int kDescBatchD = 4;
-
-template <typename W>
-__global__ void __launch_bounds__(256) k_desc_d(CacheView cv, const unsigned long long* list,
-                                                const unsigned int* list_n, unsigned int list_cap,
-                                                unsigned int implicit_atoms) {
-  using P = PathD<W, kVptD>;
-  constexpr int N = kDescBatchD;
-  __shared__ uint64_t s_d[8][N];
-  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-  ListGenD<W> gen;
-  gen.cv = &cv;
-  gen.d = s_d[wib];
-  const uint32_t warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const uint32_t nwarps = (gridDim.x * blockDim.x) >> 5;
-  unsigned n = implicit_atoms;
-  if (list) n = min(*list_n, list_cap);
-  typename P::Pending pend;
-  typename P::Ids idr;
-  for (uint32_t base = warp * N; base < n; base += nwarps * N) {
-    if (__any_sync(kFull, stop_requested(cv))) break;
-    const uint32_t cnt = min(uint32_t(N), n - base);
-    if (lane < N)
-      s_d[wib][lane] = lane < int(cnt) ? (list ? list[base + lane] : pack_desc(kAtom, base + lane, 0))
-                                       : pack_desc(kAtom, 0, 0);
-    __syncwarp();
-    P::template batch<false>(cv, gen, int(cnt), (1u << cnt) - 1u, pend, idr);
-    __syncwarp();
-  }
-  WarpDedup::flush(pend);
-  WarpDedup::retire(cv, idr);
-  if (implicit_atoms && blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(&cv.ctr->built_k[cv.kind], (unsigned long long)n);
-}
 
 // ===========================================================================
 // Batch kernels: the path-D engine over many problems at once. Work items of
@@ -2541,53 +2277,6 @@ struct LaunchC {
 };
 
 template <typename W>
-struct LaunchD {
-  static cudaError_t desc_list(const CacheView& cv, const unsigned long long* list, const unsigned int* list_n,
-                               unsigned int cap, unsigned int atoms, const LaunchCfg& lc) {
-    static int occ = occupancy_blocks((const void*)k_desc_d<W>, 256, 0);
-    const unsigned n = list ? cap : atoms;
-    const unsigned per_block = 8u * unsigned(kDescBatchD);
-    const unsigned blocks = std::max(1u, std::min((n + per_block - 1u) / per_block, unsigned(lc.sms * occ)));
-    k_desc_d<W><<<blocks, 256, 0, lc.stream>>>(cv, list, list_n, cap, atoms);
-    return cudaGetLastError();
-  }
-  static cudaError_t unary(const CacheView& cv, uint32_t first, uint32_t count, uint32_t ops, const LaunchCfg& lc) {
-    const unsigned M = cv.vecs * 16u;
-    if (cv.planes <= 1 && M >= kStagedMinBytes && M <= kStagedMaxBytes) {
-      // one block per SM holding as many warps as rows fit its shared memory
-      static int optin = [] {
-        int dev = 0, v = 0;
-        if (cudaGetDevice(&dev) != cudaSuccess ||
-            cudaDeviceGetAttribute(&v, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess)
-          v = 0;
-        return v;
-      }();
-      const int dyn_cap = optin - 1024;  // room for the kernel's static shared memory
-      const unsigned warps = dyn_cap > 0 ? std::min(unsigned(kStagedMaxWarps), unsigned(dyn_cap) / M) : 0u;
-      if (warps >= 4u) {
-        static const cudaError_t attr = cudaFuncSetAttribute((const void*)k_unary_ds<W>,
-                                                             cudaFuncAttributeMaxDynamicSharedMemorySize, dyn_cap);
-        if (attr != cudaSuccess) return attr;
-        const unsigned blocks = std::max(1u, std::min((count + warps - 1u) / warps, unsigned(lc.sms)));
-        k_unary_ds<W><<<blocks, 32u * warps, size_t(warps) * M, lc.stream>>>(cv, first, count, ops);
-        return cudaGetLastError();
-      }
-    }
-    static int occ = occupancy_blocks((const void*)k_unary_d<W>, 256, 0);
-    const unsigned blocks = std::max(1u, std::min((count + 63u) / 64u, unsigned(lc.sms * occ)));
-    k_unary_d<W><<<blocks, 256, 0, lc.stream>>>(cv, first, count, ops);
-    return cudaGetLastError();
-  }
-  static cudaError_t binary(const CacheView& cv, const BinaryPlan& plan, const LaunchCfg& lc) {
-    static int occ = occupancy_blocks((const void*)k_binary_d<W>, 256, 0);
-    const unsigned long long want = (plan.total_pairs + 63ull) / 64ull;
-    const unsigned blocks = unsigned(std::max(1ull, std::min(want, (unsigned long long)lc.sms * occ)));
-    k_binary_d<W><<<blocks, 256, 0, lc.stream>>>(cv, plan);
-    return cudaGetLastError();
-  }
-};
-
-template <typename W>
 int Kernels<W>::path_for(unsigned vecs) {
   if (vecs == 1 || vecs == 2 || vecs == 4 || vecs == 8) return 1;
   if (vecs == 32) return 2;
@@ -2603,7 +2292,7 @@ int Kernels<W>::path_for(unsigned vecs) {
     case 8: return LaunchA<W, 8>::CALL;                 \
     case 32: return LaunchC<W>::CALL;                   \
     default:                                            \
-      if (vecs > 32 && vecs % 32 == 0) return LaunchD<W>::CALL; \
+      if (vecs > 32 && vecs % 32 == 0) return GroupKernels<W>::CALL; \
       return cudaErrorInvalidValue;                     \
   }
 
