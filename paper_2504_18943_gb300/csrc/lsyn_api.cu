@@ -644,6 +644,14 @@ lsyn_status lsyn::ctx_shell(const lsyn_problem* problem, const lsyn_config* conf
   return LSYN_OK;
 }
 
+// A hash table inside a block: its buckets are read with one aligned load each
+// (an allocator of the caller's may align its blocks to less).
+constexpr size_t kBucketBytes = 32;
+static unsigned long long* table_at(void* p) {
+  const uintptr_t a = (reinterpret_cast<uintptr_t>(p) + kBucketBytes - 1) & ~uintptr_t(kBucketBytes - 1);
+  return p ? reinterpret_cast<unsigned long long*>(a) : nullptr;
+}
+
 lsyn_status lsyn::ctx_create(const lsyn_problem* problem, const lsyn_config* config, bool warp_layout,
                              lsyn_ctx** out) {
   std::vector<uint32_t> consts, atoms;
@@ -659,7 +667,7 @@ lsyn_status lsyn::ctx_create(const lsyn_problem* problem, const lsyn_config* con
   cudaError_t e;
   c->arena = static_cast<uint4*>(c->mem.get(size_t(c->max_entries) * M));
   c->prov = static_cast<unsigned long long*>(c->mem.get(size_t(c->max_entries) * 8));
-  c->table = static_cast<unsigned long long*>(c->mem.get(size_t(c->table_cap) * 8));
+  c->table = table_at(c->mem.get(size_t(c->table_cap) * 8 + kBucketBytes));
   c->ctr = static_cast<DevCounters*>(c->mem.get(sizeof(DevCounters)));
   c->consts = static_cast<uint4*>(c->mem.get(size_t(5) * M));
   c->atoms = static_cast<uint4*>(c->mem.get(size_t(c->n_props) * M));
@@ -678,7 +686,7 @@ lsyn_status lsyn::ctx_create(const lsyn_problem* problem, const lsyn_config* con
   c->big_table = c->table;
   c->big_cap = c->table_cap;
   if (c->big_cap >= 8 * lsyn_ctx::kFrontSlots) {
-    c->front_table = static_cast<unsigned long long*>(c->mem.get(size_t(lsyn_ctx::kFrontSlots) * 8));
+    c->front_table = table_at(c->mem.get(size_t(lsyn_ctx::kFrontSlots) * 8 + kBucketBytes));
     if (!c->front_table) return bail(LSYN_E_NOMEM, "device allocation failed");
     if ((e = cudaStreamCreateWithFlags(&c->side, cudaStreamNonBlocking)) != cudaSuccess)
       return bail(LSYN_E_CUDA, cudaGetErrorString(e));

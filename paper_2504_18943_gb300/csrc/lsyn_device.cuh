@@ -260,28 +260,25 @@ __device__ __forceinline__ uint4 row_op(const CacheView& cv, uint32_t op, const 
 
 
 // ---------------------------------------------------------------------------
-// Hash of a CM: over its 32-bit words w_i, H = (sum hi32(p_i), sum lo32(p_i))
-// mod 2^32 with p_i = (w_i xor key_i) * mul_i as a 64-bit product, then a
-// 64-bit finaliser. The low bits index the table, the high 32 bits are the
+// Hash of a CM over its 32-bit words w_i: 64-bit sums of w_i * mul_i (64-bit
+// products), one per 16-byte vector (paths A) or per lane of a warp (the
+// others), whose low and high halves are added up separately mod 2^32 and mixed
+// by a 64-bit finaliser. The low bits index the table, the high 32 bits are the
 // slot tag. Equal CMs always hash equally; collisions only cost a compare.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ void h_acc(uint4 v, uint4 key, uint4 mul, uint32_t& lo, uint32_t& hi) {
-  uint64_t p;
-  p = uint64_t(v.x ^ key.x) * mul.x; lo += uint32_t(p); hi += uint32_t(p >> 32);
-  p = uint64_t(v.y ^ key.y) * mul.y; lo += uint32_t(p); hi += uint32_t(p >> 32);
-  p = uint64_t(v.z ^ key.z) * mul.z; lo += uint32_t(p); hi += uint32_t(p >> 32);
-  p = uint64_t(v.w ^ key.w) * mul.w; lo += uint32_t(p); hi += uint32_t(p >> 32);
-}
-
-// Warp-path variant of the hash: acc += w_i * mul_i (64-bit products and sum)
-// per 32-bit word, then the two 32-bit halves are summed across the warp and
-// finalised with h_fin. Equal CMs hash equally; that is all dedup needs.
 __device__ __forceinline__ uint64_t h_mac(uint4 v, uint4 mul, uint64_t acc) {
   acc += uint64_t(v.x) * mul.x;
   acc += uint64_t(v.y) * mul.y;
   acc += uint64_t(v.z) * mul.z;
   acc += uint64_t(v.w) * mul.w;
   return acc;
+}
+
+// Path A: one vector's share of the two sums.
+__device__ __forceinline__ void h_acc(uint4 v, uint4 mul, uint32_t& lo, uint32_t& hi) {
+  const uint64_t acc = h_mac(v, mul, 0ull);
+  lo += uint32_t(acc);
+  hi += uint32_t(acc >> 32);
 }
 
 __device__ __forceinline__ uint64_t h_fin(uint32_t hi, uint32_t lo) {
@@ -323,33 +320,82 @@ __device__ __forceinline__ void st_release(unsigned long long* p, unsigned long 
   asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }
 
-__device__ __forceinline__ unsigned long long cas_acquire(unsigned long long* p, unsigned long long cmp,
+__device__ __forceinline__ unsigned long long cas_relaxed(unsigned long long* p, unsigned long long cmp,
                                                           unsigned long long val) {
   unsigned long long old;
-  asm volatile("atom.acquire.gpu.global.cas.b64 %0, [%1], %2, %3;" : "=l"(old) : "l"(p), "l"(cmp), "l"(val) : "memory");
+  asm volatile("atom.relaxed.gpu.global.cas.b64 %0, [%1], %2, %3;" : "=l"(old) : "l"(p), "l"(cmp), "l"(val) : "memory");
   return old;
 }
 
-__device__ __forceinline__ unsigned long long ld_acquire_u64(const unsigned long long* p) {
-  unsigned long long v;
-  asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
-  return v;
+// ---------------------------------------------------------------------------
+// Probing. A table is open-addressed with linear probing in buckets of four
+// slots (32 bytes, one sector): a CM's home is the first slot of the bucket
+// that its hash names, and the slots from there on are visited in order. A
+// probe reads a whole bucket with one 256-bit load, so that a foreign tag in the
+// way costs no round trip of its own: with single slots at a load of 0.2-0.5
+// some lane of nearly every warp needed a second and third one.
+//
+// The load has acquire semantics: when a slot's value is a published id, the
+// writer's release (fence.acq_rel.gpu, then a relaxed store of the slot)
+// synchronises with it, so the entry's CM row, stored before the release, is
+// visible to this thread's later reads, and, after a warp barrier, to its
+// warp's. The four values are four accesses in no particular order; that is
+// enough, since within a launch a slot never becomes empty again and never
+// changes hands: an empty slot that a probe stops at may have been filled
+// since, and the slots after it too, but then the claim of it fails and the
+// probe reads the bucket again.
+//
+// An empty slot is claimed with a compare-and-swap, relaxed: a claim that
+// loses reads its bucket again (with acquire) before it does anything else.
+// Reading first keeps the atomics to the inserts: most probes meet an equal
+// CM, and on this GPU a random load costs far less than a random atomic.
+// ---------------------------------------------------------------------------
+__host__ __device__ __forceinline__ unsigned long long home_slot(unsigned long long h, unsigned long long mask) {
+  return h & mask & ~3ull;
 }
 
-// One probe of a table slot: returns what is there, after claiming the slot
-// with `val` if it was empty (then 0). The slot is read first and claimed with
-// a compare-and-swap only when it reads empty: most probes meet an occupied
-// slot (an equal CM, or another tag), and on this GPU a random load costs far
-// less than a random atomic (whole solves 1.45x faster than one CAS per probe).
-// A claim that loses a race returns the winner's value, as the CAS alone
-// would. Acquire semantics (load and CAS): when the value is a published id,
-// the writer's release (fence.acq_rel.gpu, then a relaxed store of the slot)
-// synchronises with this read, so the entry's CM row, stored before the
-// release, is visible to this thread's later reads, and, after a warp
-// barrier, to its warp's.
-__device__ __forceinline__ unsigned long long probe_slot(unsigned long long* p, unsigned long long val) {
-  const unsigned long long sv = ld_acquire_u64(p);
-  return sv != 0ull ? sv : cas_acquire(p, 0ull, val);
+enum : int { kSeeEmpty = 0, kSeeFull = 1, kSeePending = 2, kSeeMatch = 3, kSeeNothing = 4 };
+
+// From slot `pos` to the end of its bucket: the first slot that is empty,
+// a tombstone or has this tag (the high word of the hash), with pos moved to it
+// and id1 = id + 1 for a published entry; kSeeNothing, with pos moved to the
+// next bucket, if there is none. A tombstone is left only by a claim past a
+// full arena, and such a level is incomplete: the candidate could not be
+// inserted any more, so probing stops there (kSeeFull; a small table full of
+// tombstones would otherwise leave it nowhere to stop).
+__device__ __forceinline__ int see_bucket(const unsigned long long* table, unsigned long long mask,
+                                          unsigned long long& pos, uint32_t tag, uint32_t& id1) {
+  const unsigned long long w = pos & ~3ull;
+  unsigned long long s[4];
+  asm volatile("ld.acquire.gpu.global.v4.u64 {%0, %1, %2, %3}, [%4];"
+               : "=l"(s[0]), "=l"(s[1]), "=l"(s[2]), "=l"(s[3])
+               : "l"(table + w)
+               : "memory");
+  uint32_t stops = 0;  // bit k: slot k ends the probe (an empty slot is 0, its low word suffices)
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const uint32_t lo = uint32_t(s[k]);
+    stops |= lo == 0u || lo == kSlotTomb || uint32_t(s[k] >> 32) == tag ? 1u << k : 0u;
+  }
+  stops &= 15u << unsigned(pos & 3ull);
+  if (stops == 0u) {
+    id1 = 0u;
+    pos = (w + 4ull) & mask;
+    return kSeeNothing;
+  }
+  const int at = __ffs(stops) - 1;
+  const uint32_t low = at < 2 ? (at == 0 ? uint32_t(s[0]) : uint32_t(s[1])) : (at == 2 ? uint32_t(s[2]) : uint32_t(s[3]));
+  id1 = low;
+  pos = w + unsigned(at);
+  return low == 0u ? kSeeEmpty : low == kSlotTomb ? kSeeFull : low == kSlotPending ? kSeePending : kSeeMatch;
+}
+
+// Claims an empty slot: 0 if it did, 1 if an equal tag was first and is still
+// pending (a candidate with this hash), 2 if the bucket has to be read again.
+__device__ __forceinline__ int claim_slot(unsigned long long* slot, uint32_t tag) {
+  const unsigned long long mine = ((unsigned long long)tag << 32) | kSlotPending;
+  const unsigned long long was = cas_relaxed(slot, 0ull, mine);
+  return was == 0ull ? 0 : was == mine ? 1 : 2;
 }
 
 __device__ __forceinline__ unsigned ld_relaxed_u32(const unsigned* p) {
@@ -393,40 +439,40 @@ __device__ __forceinline__ const uint4* row_ptr(const CacheView& cv, uint32_t id
 }
 
 // Pair `local` of a split, as row offsets (left, right). For a level paired
-// with itself: the pairs a < b in order of b (b = 1, 2, ...; a = 0 .. b-1), so
-// that no pair index is wasted. Otherwise, with large_outer, the right
-// (larger) side's rows in order, each with every row of the left (smaller)
-// side: each large row is read once while the small side stays in L2, which
-// made 16 KiB CMs (path D) 15 % faster at the large workload's level 8 than
-// the left-major order; without it, row-major over left x right, which
-// measured faster for CMs of up to 128 bytes (path A), whose levels L2 holds
-// anyway.
+// with itself: the pairs a < b, those of b = n - 1 - r and of b = r (n - 1
+// together) after one another for r = 0, 1, ..., so that no pair index is wasted
+// and one division finds a pair (the inverse of a triangular count takes a
+// double-precision square root, which this GPU computes at a small fraction of
+// its other rates). Otherwise, with large_outer, the right (larger) side's rows
+// in order, each with every row of the left (smaller) side: each large row is
+// read once while the small side stays in L2; without it, row-major over left x
+// right, which measured faster for CMs of up to 128 bytes (path A), whose
+// levels L2 holds anyway.
 __device__ __forceinline__ uint2 split_pair(const Split& S, unsigned long long local, bool large_outer) {
-  if (!S.tri) {
-    if ((local >> 32) == 0ull) {  // the usual case: a 32-bit division
-      const uint32_t l = uint32_t(local), n = large_outer ? S.left_n : S.right_n, q = l / n;
-      return large_outer ? make_uint2(l - q * n, q) : make_uint2(q, l - q * n);
-    }
-    if (large_outer) {
-      const uint32_t ib = uint32_t(local / S.left_n);
-      return make_uint2(uint32_t(local - (unsigned long long)ib * S.left_n), ib);
-    }
-    const uint32_t ia = uint32_t(local / S.right_n);
-    return make_uint2(ia, uint32_t(local - (unsigned long long)ia * S.right_n));
+  const uint32_t n = S.tri ? S.left_n - 1u : large_outer ? S.left_n : S.right_n;
+  uint32_t q, r;
+  if ((local >> 32) == 0ull) {  // the usual case: a 32-bit division
+    q = uint32_t(local) / n;
+    r = uint32_t(local) - q * n;
+  } else {
+    q = uint32_t(local / n);
+    r = uint32_t(local - (unsigned long long)q * n);
   }
-  unsigned long long b = (unsigned long long)((1.0 + sqrt(1.0 + 8.0 * double(local))) * 0.5);
-  while (b > 1 && b * (b - 1) / 2 > local) --b;
-  while ((b + 1) * b / 2 <= local) ++b;
-  return make_uint2(uint32_t(local - b * (b - 1) / 2), uint32_t(b));
+  if (S.tri) {
+    const uint32_t b = n - q;  // n is the last row
+    return r < b ? make_uint2(r, b) : make_uint2(r - b, q);
+  }
+  return large_outer ? make_uint2(r, q) : make_uint2(q, r);
 }
 
 // ===========================================================================
-// Path A: one thread holds a whole CM (V vectors, at most 128 bytes).
+// Path A of the batch kernels: one thread holds a whole CM (V vectors, at most
+// 128 bytes).
 // ===========================================================================
 template <typename W, int V>
 struct PathA {
   struct Consts {
-    uint4 lm[V], lab[V], care[V], key[V], mul[V];
+    uint4 lm[V], lab[V], care[V], mul[V];
   };
 
   __device__ static void load_consts(const CacheView& cv, Consts* s) {
@@ -434,7 +480,6 @@ struct PathA {
       s->lm[i] = cv.lenmask[i];
       s->lab[i] = cv.label[i];
       s->care[i] = cv.care[i];
-      s->key[i] = cv.hkey[i];
       s->mul[i] = cv.hmul[i];
     }
   }
@@ -451,47 +496,45 @@ struct PathA {
     uint32_t lo = 0, hi = 0, bad = 0;
 #pragma unroll
     for (int v = 0; v < V; ++v) {
-      h_acc(c[v], s.key[v], s.mul[v], lo, hi);
+      h_acc(c[v], s.mul[v], lo, hi);
       bad |= spec_bad(c[v], s.lab[v], s.care[v]);
     }
     if (bad == 0) record_solution(cv, desc);
     if (full) return 0;
     const uint64_t h = h_fin(hi, lo);
-    const unsigned long long tag = (h >> 32) << 32;
-    unsigned long long pos = h & cv.table_mask;
-    for (unsigned long long it = 0; it <= cv.table_mask; ++it, pos = (pos + 1) & cv.table_mask) {
-      unsigned long long* slot = cv.table + pos;
-      // Claims an empty slot, or returns what is there.
-      const unsigned long long sv = probe_slot(slot, tag | kSlotPending);
-      if (sv == 0ull) {
-        const unsigned id = atomicAdd(&cv.ctr->n_entries, 1u);
-        if (id >= cv.max_entries) {
-          st_release(slot, tag | kSlotTomb);
-          atomicExch(&cv.ctr->full, 1u);
-          return 0;
-        }
-        uint4* dst = cv.arena + size_t(id) * cv.vecs;
+    const uint32_t tag = uint32_t(h >> 32);
+    unsigned long long pos = home_slot(h, cv.table_mask);
+    for (unsigned long long it = 0; it <= cv.table_mask; ++it) {
+      uint32_t id1;
+      const int saw = see_bucket(cv.table, cv.table_mask, pos, tag, id1);
+      if (saw == kSeeFull) return 0;
+      if (saw == kSeePending) { defer(cv, desc); return 0; }
+      if (saw == kSeeMatch) {
+        const uint4* src = row_ptr(cv, id1 - 1u);
+        uint32_t ne = 0;
 #pragma unroll
-        for (int v = 0; v < V; ++v) dst[v] = c[v];
-        cv.prov[id] = desc;
-        cv.slotpos[id] = unsigned(pos);
-        cv.homes[id] = uint32_t(h);
-        st_release(slot, tag | (unsigned long long)(id + 1u));  // orders this thread's CM and provenance first
-        return 1;
+        for (int v = 0; v < V; ++v) ne |= v_ne(__ldcg(src + v), c[v]);
+        if (ne == 0) return 0;  // duplicate: an equal CM is already cached
+        pos = (pos + 1) & cv.table_mask;
       }
-      // A tombstone is left only by a claim past a full arena, and such a
-      // level is incomplete: the candidate could not be inserted any more,
-      // so probing stops (a small table full of tombstones would otherwise
-      // leave it nowhere to stop).
-      if (uint32_t(sv) == kSlotTomb) return 0;
-      if ((sv & 0xFFFFFFFF00000000ull) != tag) continue;
-      const uint32_t low = uint32_t(sv);
-      if (low == kSlotPending) { defer(cv, desc); return 0; }
-      const uint4* src = row_ptr(cv, low - 1u);
-      uint32_t ne = 0;
+      if (saw != kSeeEmpty) continue;
+      unsigned long long* slot = cv.table + pos;
+      if (claim_slot(slot, tag) != 0) continue;
+      const unsigned id = atomicAdd(&cv.ctr->n_entries, 1u);
+      const unsigned long long tag64 = (unsigned long long)tag << 32;
+      if (id >= cv.max_entries) {
+        st_release(slot, tag64 | kSlotTomb);
+        atomicExch(&cv.ctr->full, 1u);
+        return 0;
+      }
+      uint4* dst = cv.arena + size_t(id) * cv.vecs;
 #pragma unroll
-      for (int v = 0; v < V; ++v) ne |= v_ne(__ldcg(src + v), c[v]);
-      if (ne == 0) return 0;  // duplicate: an equal CM is already cached
+      for (int v = 0; v < V; ++v) dst[v] = c[v];
+      cv.prov[id] = desc;
+      cv.slotpos[id] = unsigned(pos);
+      cv.homes[id] = uint32_t(h);
+      st_release(slot, tag64 | (unsigned long long)(id + 1u));  // orders this thread's CM and provenance first
+      return 1;
     }
     atomicExch(&cv.ctr->error, 1u);
     return 0;
@@ -505,61 +548,6 @@ struct PathA {
     return process(cv, s, c, desc, full);
   }
 };
-
-template <typename W, int V>
-__global__ void __launch_bounds__(256) k_unary_a(CacheView cv, uint32_t first, uint32_t count, uint32_t ops) {
-  using P = PathA<W, V>;
-  __shared__ typename P::Consts s;
-  P::load_consts(cv, &s);
-  __syncthreads();
-  unsigned long long built = 0, ins = 0;
-  const uint32_t stride = gridDim.x * blockDim.x;
-  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < count; i += stride) {
-    if (stop_requested(cv)) break;
-    const bool full = ld_relaxed_u32(&cv.ctr->full) != 0u;
-    const uint32_t id = first + i;
-    uint4 a[V];
-    P::load_row(row_ptr(cv, id), a);
-    const uint32_t opc[4] = {kNot, kNext, kFuture, kGlobally};
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      if (!((ops >> q) & 1u)) continue;
-      ins += P::candidate(cv, s, opc[q], a, a, pack_desc(opc[q], id, 0), full);
-      ++built;
-    }
-  }
-  if (built) atomicAdd(&cv.ctr->built_k[cv.kind], built);
-  if (ins) atomicAdd(&cv.ctr->inserted_k[cv.kind], ins);
-}
-
-template <typename W, int V>
-__global__ void __launch_bounds__(256) k_binary_a(CacheView cv, BinaryPlan plan) {
-  using P = PathA<W, V>;
-  __shared__ typename P::Consts s;
-  P::load_consts(cv, &s);
-  __syncthreads();
-  unsigned long long built = 0, ins = 0;
-  const unsigned long long stride = (unsigned long long)gridDim.x * blockDim.x;
-  for (unsigned long long p = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; p < plan.total_pairs;
-       p += stride) {
-    if (stop_requested(cv)) break;
-    int sp = 0;
-    while (sp + 1 < plan.n_splits && plan.s[sp + 1].pairs_begin <= p) ++sp;
-    const Split& S = plan.s[sp];
-    const uint2 ab = split_pair(S, p - S.pairs_begin, false);
-    const uint32_t a_id = S.left_start + ab.x, b_id = S.right_start + ab.y;
-    const bool full = ld_relaxed_u32(&cv.ctr->full) != 0u;
-    uint4 a[V], b[V];
-    P::load_row(row_ptr(cv, a_id), a);
-    P::load_row(row_ptr(cv, b_id), b);
-    if (plan.ops & 1u) { ins += P::candidate(cv, s, kAnd, a, b, pack_desc(kAnd, a_id, b_id), full); ++built; }
-    if (plan.ops & 2u) { ins += P::candidate(cv, s, kOr, a, b, pack_desc(kOr, a_id, b_id), full); ++built; }
-    if (plan.ops & 4u) { ins += P::candidate(cv, s, kUntil, a, b, pack_desc(kUntil, a_id, b_id), full); ++built; }
-    if (plan.ops & 8u) { ins += P::candidate(cv, s, kUntil, b, a, pack_desc(kUntil, b_id, a_id), full); ++built; }
-  }
-  if (built) atomicAdd(&cv.ctr->built_k[cv.kind], built);
-  if (ins) atomicAdd(&cv.ctr->inserted_k[cv.kind], ins);
-}
 
 // Rebuild a candidate from its descriptor (operands are complete levels).
 template <typename W, int V>
@@ -578,29 +566,6 @@ __device__ void rebuild_a(const CacheView& cv, const typename PathA<W, V>::Const
   }
 #pragma unroll
   for (int v = 0; v < V; ++v) c[v] = v_op<W>(op, a[v], b[v], s.lm[v], cv.steps);
-}
-
-template <typename W, int V>
-__global__ void __launch_bounds__(256) k_desc_a(CacheView cv, const unsigned long long* list,
-                                                const unsigned int* list_n, unsigned int list_cap,
-                                                unsigned int implicit_atoms) {
-  using P = PathA<W, V>;
-  __shared__ typename P::Consts s;
-  P::load_consts(cv, &s);
-  __syncthreads();
-  unsigned n = implicit_atoms;
-  if (list) n = min(*list_n, list_cap);
-  const uint32_t stride = gridDim.x * blockDim.x;
-  unsigned long long ins = 0;
-  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
-    if (stop_requested(cv)) break;
-    const uint64_t d = list ? list[i] : pack_desc(kAtom, i, 0);
-    uint4 c[V];
-    rebuild_a<W, V>(cv, s, d, c);
-    ins += P::process(cv, s, c, d, ld_relaxed_u32(&cv.ctr->full) != 0u);
-  }
-  if (ins) atomicAdd(&cv.ctr->inserted_k[cv.kind], ins);
-  if (implicit_atoms && blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(&cv.ctr->built_k[cv.kind], (unsigned long long)n);
 }
 
 // ===========================================================================
@@ -649,14 +614,18 @@ struct WarpDedup {
     unsigned pre = 0;
     bool pre_ok = false;
     unsigned long long inserted = 0;
+    unsigned polls = 0;  // of the arena-full flag
+    bool full = false;   // the arena is full
   };
 
-  // The arena-full flag, polled by every batch: once the arena is full each
-  // further claim leaves a tombstone in the table, so warps must stop
-  // claiming at once (a flag polled every few batches let the tombstones of
-  // a small table fill it). The flag has a cache line of its own.
-  __device__ static bool arena_full(const CacheView& cv) {
-    return __any_sync(kFull, (threadIdx.x & 31) == 0 && ld_relaxed_u32(&cv.ctr->full) != 0u);
+  // Whether the arena is full (then further claims would only leave
+  // tombstones in the table). A warp whose own claims found no id left stops
+  // claiming at once; the flag that tells it of the others' is polled every
+  // fourth batch only, since every warp's polls go to one L2 slice.
+  __device__ static bool arena_full(const CacheView& cv, Ids& ids) {
+    if ((ids.polls++ & 3u) == 0u)
+      ids.full = ids.full || __any_sync(kFull, (threadIdx.x & 31) == 0 && ld_relaxed_u32(&cv.ctr->full) != 0u);
+    return ids.full;
   }
 
   __device__ static void prefetch(const CacheView& cv, Ids& ids) {
@@ -706,6 +675,8 @@ struct WarpDedup {
     ids.next = ids.end = 0;
     ids.pre_ok = false;
     ids.inserted = 0;
+    ids.polls = 0;
+    ids.full = false;
   }
 
   // A slot this lane claimed whose CM words were stored but not yet
@@ -816,13 +787,13 @@ struct PathC {
     // Once the arena is full this level can never be extended: only the spec
     // check (above) matters, so the rest of the batch skips the dedup instead
     // of filling the table with tombstones.
-    const bool full = WarpDedup::arena_full(cv);
+    const bool full = WarpDedup::arena_full(cv, ids);
     int state = (mine && !full) ? WarpDedup::kProbing : WarpDedup::kDone;
     constexpr int kProbing = WarpDedup::kProbing, kDone = WarpDedup::kDone,
                   kClaimed = WarpDedup::kClaimed, kDeferred = WarpDedup::kDeferred;
     const uint64_t h = h_fin(my_hi, my_lo);
     const unsigned long long tag = (h >> 32) << 32;
-    unsigned long long pos = h & cv.table_mask;
+    unsigned long long pos = home_slot(h, cv.table_mask);
 
     // Twins inside the batch (equal hashes; common, since the batch's
     // candidates share an operand): compare each with its lowest-lane twin in
@@ -842,21 +813,19 @@ struct PathC {
     uint32_t cmp_id = 0;
     unsigned long long guard = 0;
     while (true) {
+      // Read the buckets; then claims of empty slots and compares, in flight
+      // together. A lost claim reads its bucket again in the next round.
       bool need = false;
+      int claim = 2;
       if (state == kProbing) {
-        // Claims an empty slot, or returns what is there.
-        const unsigned long long sv = probe_slot(cv.table + pos, tag | kSlotPending);
-        if (sv == 0ull) {
-          state = kClaimed;
-        } else {
-          const uint32_t low = uint32_t(sv);
-          if (low == kSlotTomb) state = kDone;  // the arena is full: this level is incomplete (see path A)
-          else if ((sv & 0xFFFFFFFF00000000ull) != tag) pos = (pos + 1) & cv.table_mask;
-          else if (low == kSlotPending) state = kDeferred;
-          else {
-            need = true;
-            cmp_id = low - 1u;
-          }
+        uint32_t id1;
+        const int saw = see_bucket(cv.table, cv.table_mask, pos, uint32_t(tag >> 32), id1);
+        if (saw == kSeeEmpty) claim = claim_slot(cv.table + pos, uint32_t(tag >> 32));
+        else if (saw == kSeeFull) state = kDone;  // the arena is full
+        else if (saw == kSeePending) state = kDeferred;
+        else if (saw == kSeeMatch) {
+          need = true;
+          cmp_id = id1 - 1u;
         }
       }
       uint32_t cm = __ballot_sync(kFull, need);
@@ -885,6 +854,7 @@ struct PathC {
           else pos = (pos + 1) & cv.table_mask;
         }
       }
+      if (claim < 2) state = claim == 0 ? kClaimed : kDeferred;
       if (!__any_sync(kFull, state == kProbing)) break;
       if (++guard > cv.table_mask) {  // every slot seen: cannot happen at load <= 0.9
         if (lane == 0) atomicExch(&cv.ctr->error, 1u);
@@ -911,7 +881,9 @@ struct PathC {
       const unsigned my_rank = unsigned(__popc(claim & ((1u << lane) - 1u)));
       const unsigned my_id = my_rank < have ? ids.next + my_rank : fresh + (my_rank - have);
       WarpDedup::advance(cv, ids, n_claim, have, fresh, use_pre, last);
-      ids.inserted += __popc(__ballot_sync(kFull, state == kClaimed && my_id < cv.max_entries));
+      const unsigned wrote = unsigned(__popc(__ballot_sync(kFull, state == kClaimed && my_id < cv.max_entries)));
+      ids.inserted += wrote;
+      ids.full = ids.full || wrote < n_claim;
       if (state == kClaimed) {
         unsigned long long* slot = cv.table + pos;
         if (my_id < cv.max_entries) {
@@ -1321,11 +1293,11 @@ struct PathD {
 
     constexpr int kProbing = WarpDedup::kProbing, kDone = WarpDedup::kDone,
                   kClaimed = WarpDedup::kClaimed, kDeferred = WarpDedup::kDeferred;
-    const bool full = WarpDedup::arena_full(cv);
+    const bool full = WarpDedup::arena_full(cv, ids);
     int state = (mine && !full) ? kProbing : kDone;  // a full arena: spec check only
     const uint64_t h = h_fin(my_hi, my_lo);
     const unsigned long long tag = (h >> 32) << 32;
-    unsigned long long pos = h & cv.table_mask;
+    unsigned long long pos = home_slot(h, cv.table_mask);
     // in-batch twins (equal hashes): settle them by comparing the candidates
     const uint32_t mine_mask = __ballot_sync(kFull, mine);
     const uint32_t peers = __match_any_sync(kFull, (unsigned long long)h) & mine_mask;
@@ -1343,20 +1315,19 @@ struct PathD {
     uint32_t cmp_id = 0;
     unsigned long long guard = 0;
     while (true) {
+      // Read the buckets; then claims of empty slots and compares, in flight
+      // together. A lost claim reads its bucket again in the next round.
       bool need = false;
+      int claim = 2;
       if (state == kProbing) {
-        const unsigned long long sv = probe_slot(cv.table + pos, tag | kSlotPending);
-        if (sv == 0ull) {
-          state = kClaimed;
-        } else {
-          const uint32_t low = uint32_t(sv);
-          if (low == kSlotTomb) state = kDone;  // the arena is full: this level is incomplete (see path A)
-          else if ((sv & 0xFFFFFFFF00000000ull) != tag) pos = (pos + 1) & cv.table_mask;
-          else if (low == kSlotPending) state = kDeferred;
-          else {
-            need = true;
-            cmp_id = low - 1u;
-          }
+        uint32_t id1;
+        const int saw = see_bucket(cv.table, cv.table_mask, pos, uint32_t(tag >> 32), id1);
+        if (saw == kSeeEmpty) claim = claim_slot(cv.table + pos, uint32_t(tag >> 32));
+        else if (saw == kSeeFull) state = kDone;  // the arena is full
+        else if (saw == kSeePending) state = kDeferred;
+        else if (saw == kSeeMatch) {
+          need = true;
+          cmp_id = id1 - 1u;
         }
       }
       const uint32_t need_m = __ballot_sync(kFull, need);
@@ -1388,6 +1359,7 @@ struct PathD {
         if (!((ne_m >> lane) & 1u)) state = kDone;  // equal CM already cached
         else pos = (pos + 1) & cv.table_mask;
       }
+      if (claim < 2) state = claim == 0 ? kClaimed : kDeferred;
       if (!__any_sync(kFull, state == kProbing)) break;
       if (++guard > cv.table_mask) {
         if (lane == 0) atomicExch(&cv.ctr->error, 1u);
@@ -1429,7 +1401,9 @@ struct PathD {
       const unsigned my_rank = unsigned(__popc(claim & ((1u << lane) - 1u)));
       const unsigned my_id = my_rank < have ? ids.next + my_rank : fresh + (my_rank - have);
       WarpDedup::advance(cv, ids, n_claim, have, fresh, use_pre);
-      ids.inserted += __popc(__ballot_sync(kFull, state == kClaimed && my_id < cv.max_entries));
+      const unsigned wrote = unsigned(__popc(__ballot_sync(kFull, state == kClaimed && my_id < cv.max_entries)));
+      ids.inserted += wrote;
+      ids.full = ids.full || wrote < n_claim;
       if (state == kClaimed) {
         unsigned long long* slot = cv.table + pos;
         if (my_id < cv.max_entries) {
@@ -1612,8 +1586,7 @@ __device__ __forceinline__ void batch_a_load(const CacheView& cv, uint4* ca) {
     ca[i] = cv.lenmask[i];
     ca[V + i] = cv.label[i];
     ca[2 * V + i] = cv.care[i];
-    ca[3 * V + i] = cv.hkey[i];
-    ca[4 * V + i] = cv.hmul[i];
+    ca[3 * V + i] = cv.hmul[i];
   }
   __syncwarp();
 }
@@ -1639,7 +1612,7 @@ __global__ void __launch_bounds__(256) k_batch_run(StepHeader* hdr, const StepPr
   __shared__ CacheView s_cv[8];
   __shared__ uint2 s_pairs[8][8];
   __shared__ uint64_t s_d[8][32];
-  __shared__ uint4 s_ca[8][40];  // path-A constants of the warp's problem (5 x up to 8 vectors)
+  __shared__ uint4 s_ca[8][32];  // path-A constants of the warp's problem (4 x up to 8 vectors)
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
   CacheView* cv = &s_cv[wib];
   uint4* ca = s_ca[wib];
@@ -2069,7 +2042,7 @@ static __global__ void __launch_bounds__(256) k_rehash(const unsigned long long*
     if (v == 0ull || low >= kSlotTomb) continue;
     const uint32_t id = low - 1u;
     if (id >= live_end) continue;
-    unsigned long long pos = homes[id] & new_mask;
+    unsigned long long pos = home_slot(homes[id], new_mask);
     unsigned long long it = 0;
     for (; it <= new_mask; ++it, pos = (pos + 1) & new_mask)
       if (atomicCAS(new_t + pos, 0ull, v) == 0ull) break;
@@ -2147,30 +2120,6 @@ inline int occupancy_blocks(const void* fn, int threads, size_t smem) {
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, fn, threads, smem) != cudaSuccess || n < 1) n = 1;
   return n;
 }
-
-template <typename W, int V>
-struct LaunchA {
-  static cudaError_t desc_list(const CacheView& cv, const unsigned long long* list, const unsigned int* list_n,
-                               unsigned int cap, unsigned int atoms, const LaunchCfg& lc) {
-    const unsigned n = list ? cap : atoms;
-    const unsigned blocks = std::max(1u, std::min((n + 255u) / 256u, unsigned(lc.sms * 8)));
-    k_desc_a<W, V><<<blocks, 256, 0, lc.stream>>>(cv, list, list_n, cap, atoms);
-    return cudaGetLastError();
-  }
-  static cudaError_t unary(const CacheView& cv, uint32_t first, uint32_t count, uint32_t ops, const LaunchCfg& lc) {
-    static int occ = occupancy_blocks((const void*)k_unary_a<W, V>, 256, 0);
-    const unsigned blocks = std::max(1u, std::min((count + 255u) / 256u, unsigned(lc.sms * occ)));
-    k_unary_a<W, V><<<blocks, 256, 0, lc.stream>>>(cv, first, count, ops);
-    return cudaGetLastError();
-  }
-  static cudaError_t binary(const CacheView& cv, const BinaryPlan& plan, const LaunchCfg& lc) {
-    static int occ = occupancy_blocks((const void*)k_binary_a<W, V>, 256, 0);
-    const unsigned long long want = (plan.total_pairs + 255ull) / 256ull;
-    const unsigned blocks = unsigned(std::max(1ull, std::min(want, (unsigned long long)lc.sms * occ)));
-    k_binary_a<W, V><<<blocks, 256, 0, lc.stream>>>(cv, plan);
-    return cudaGetLastError();
-  }
-};
 
 template <typename W>
 struct LaunchC {
@@ -2286,10 +2235,10 @@ int Kernels<W>::path_for(unsigned vecs) {
 
 #define LSYN_DISPATCH(vecs, CALL)                       \
   switch (vecs) {                                       \
-    case 1: return LaunchA<W, 1>::CALL;                 \
-    case 2: return LaunchA<W, 2>::CALL;                 \
-    case 4: return LaunchA<W, 4>::CALL;                 \
-    case 8: return LaunchA<W, 8>::CALL;                 \
+    case 1:                                             \
+    case 2:                                             \
+    case 4:                                             \
+    case 8: return LaneKernels<W>::CALL;                \
     case 32: return LaunchC<W>::CALL;                   \
     default:                                            \
       if (vecs > 32 && vecs % 32 == 0) return GroupKernels<W>::CALL; \

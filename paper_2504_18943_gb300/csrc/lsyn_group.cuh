@@ -15,9 +15,8 @@
 //
 // Per item: (1) every thread hashes its columns of the candidates and checks
 // the specification; (2) warp 0 adds the partial hashes up, publishes what the
-// group claimed before and claims table slots (one lane per candidate; a
-// compare-and-swap at once: these rates are far below the one at which atomics
-// queue, and a read before it would be a round trip more); (3) every thread
+// group claimed before, probes and claims table slots (one lane per candidate);
+// (3) every thread
 // compares its columns with the stored rows that the probes found, while warp 0
 // reserves ids, then writes the claimed rows and fetches its part of the next
 // item's operands. A candidate that meets a pending slot with its own tag is
@@ -419,7 +418,7 @@ __global__ void __launch_bounds__(256, group_blocks(MP)) k_group(CacheView cv, G
       const bool is_full = __any_sync(kFull, full);  // a full arena: the specification check only
       state = mine && !is_full ? kProbing : kDone;
       h = h_fin(my_hi, my_lo);
-      pos = h & cv.table_mask;
+      pos = home_slot(h, cv.table_mask);
       // twins inside the item (equal hashes): compared with the lowest one from
       // their operands, without a probe of their own
       const uint32_t mine_m = __ballot_sync(kFull, mine);
@@ -437,19 +436,20 @@ __global__ void __launch_bounds__(256, group_blocks(MP)) k_group(CacheView cv, G
       unsigned fresh = 0;
       uint32_t claimed = 0;
       if (w == 0) {
-        const unsigned long long tag = (h >> 32) << 32;
         uint32_t cmp_id = 0;
         while (__any_sync(kFull, state == kProbing)) {
           if (state == kProbing) {
-            const unsigned long long sv = cas_acquire(cv.table + pos, 0ull, tag | kSlotPending);
-            const uint32_t low = uint32_t(sv);
-            if (sv == 0ull) state = kClaimed;
-            else if (low == kSlotTomb) state = kDone;  // the arena is full: this level is incomplete (see path A)
-            else if ((sv & 0xFFFFFFFF00000000ull) != tag) pos = (pos + 1) & cv.table_mask;
-            else if (low == kSlotPending) state = kWait;
-            else {
+            uint32_t id1;
+            const int saw = see_bucket(cv.table, cv.table_mask, pos, uint32_t(h >> 32), id1);
+            if (saw == kSeeEmpty) {
+              const int claim = claim_slot(cv.table + pos, uint32_t(h >> 32));
+              if (claim < 2) state = claim == 0 ? kClaimed : kWait;
+            }
+            else if (saw == kSeeFull) state = kDone;  // the arena is full
+            else if (saw == kSeePending) state = kWait;
+            else if (saw == kSeeMatch) {
               state = kCompare;
-              cmp_id = low - 1u;
+              cmp_id = id1 - 1u;
             }
           }
           if (++guard > cv.table_mask) {  // every slot seen: cannot happen at load <= 0.9

@@ -221,6 +221,15 @@ struct Kernels {
                           const int4* nodes, int n_nodes, int steps, W* scratch, W* out, const LaunchCfg& lc);
 };
 
+// Level kernels for CMs of at most 128 bytes (lsyn_lanes.cuh).
+template <typename W>
+struct LaneKernels {
+  static cudaError_t desc_list(const CacheView& cv, const unsigned long long* list, const unsigned int* list_n,
+                               unsigned int list_cap, unsigned int implicit_atoms, const LaunchCfg& lc);
+  static cudaError_t unary(const CacheView& cv, uint32_t first, uint32_t count, uint32_t ops, const LaunchCfg& lc);
+  static cudaError_t binary(const CacheView& cv, const BinaryPlan& plan, const LaunchCfg& lc);
+};
+
 // Level kernels for CMs above 512 bytes, several warps to a candidate
 // (lsyn_group.cuh).
 template <typename W>

@@ -1,0 +1,72 @@
+"""GPU tests of the path-A level kernels (matrices of at most 128 bytes, held
+by 1, 2, 4 or 8 lanes): complete levels equal the oracle's at each width, word
+type and an odd number of traces, deep enough that warps take many batches, and
+an arena with exactly the room that the levels need is filled without loss."""
+from __future__ import annotations
+
+import numpy as np
+import pytest
+
+import oracle
+from paper_2504_18943_gb300 import workloads as W
+from tests import gpu_util as U
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def L():
+    return U.lib()
+
+
+def _problem(props, traces, lo, hi, bits, seed=7):
+    tb = W.draw_traces(W.Stream(W.stream_key(seed, 6)), traces, props, lo, hi, np.full(props, 0.5))
+    return W.Problem("lanes", props, tb, traces // 2, traces - traces // 2, bits)
+
+
+CASES = [
+    (2, 3, 5, 32, 32, 9, 0x7F),     # one vector
+    (2, 2, 20, 64, 64, 9, 0x5B),
+    (3, 7, 6, 32, 32, 7, 0x7F),     # two vectors
+    (2, 14, 6, 6, 32, 10, 0x5B),    # four vectors, the paper's grammar
+    (3, 8, 8, 64, 64, 7, 0x7F),
+    (4, 30, 8, 32, 32, 7, 0x7F),    # eight vectors
+    (3, 15, 8, 64, 64, 7, 0x2D),    # not, or, X, G
+    (1, 32, 1, 32, 32, 11, 0x7F),
+]
+
+
+@pytest.mark.parametrize("props,traces,lo,hi,bits,depth,ops", CASES)
+def test_levels_equal_the_oracle(L, props, traces, lo, hi, bits, depth, ops):
+    p = _problem(props, traces, lo, hi, bits)
+    run = oracle.Spec.from_problem(p).enumerate(depth, ops)
+    with L.Synthesizer(L.pack_problem(p), L.torch_config(op_mask=ops, cache_bytes=1 << 30, full_levels=True)) as s:
+        for k in range(1, depth + 1):
+            st = s.level(k)
+            assert st.unique == run.size(k), k
+            want = U.sorted_rows(U.oracle_level_words(run, k, p.traces.lengths, bits))
+            assert np.array_equal(U.sorted_rows(s.export(k)), want), k
+
+
+def _bytes_for(entries, row):
+    """cache_bytes whose arena holds exactly `entries` rows (a table at most
+    half full beside them, 16 bytes of records an entry)."""
+    cap = 1024
+    while cap // 2 < entries:
+        cap *= 2
+    return cap * 8 + entries * (row + 16)
+
+
+@pytest.mark.parametrize("traces,bits,row,depth", [(4, 32, 16, 9), (14, 32, 64, 9), (30, 32, 128, 9)])
+def test_arena_of_exactly_the_levels_size(L, traces, bits, row, depth):
+    """As many entries as levels 1..depth hold: the last level is complete. One
+    fewer: it is not, and says so."""
+    p = L.pack_problem(_problem(2, traces, 6, 24, bits))
+    with L.Synthesizer(p, L.torch_config(cache_bytes=1 << 30, full_levels=True)) as s:
+        sizes = [s.level(k).unique for k in range(1, depth + 1)]
+    total = sum(sizes)
+    for room, full in ((total, 0), (total - 1, 1)):
+        with L.Synthesizer(p, L.make_config(cache_bytes=_bytes_for(room, row), full_levels=True)) as s:
+            got = [s.level(k) for k in range(1, depth + 1)]
+        assert [st.unique for st in got[:-1]] == sizes[:-1]
+        assert got[-1].cache_full == full and got[-1].unique == sizes[-1] - full
