@@ -10,6 +10,7 @@
 // few counters back per level.
 #include <algorithm>
 #include <chrono>
+#include <cstddef>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
@@ -20,6 +21,7 @@
 #include "lsyn.h"
 #include "lsyn_ctx.h"
 #include "lsyn_internal.h"
+#include "lsyn_text.cuh"
 
 using namespace lsyn;
 
@@ -71,67 +73,16 @@ __global__ void k_level_begin(DevCounters* c) {
   c->sol = ~0ull;
 }
 
-__device__ void reconstruct_one(const unsigned long long* prov, unsigned long long root,
-                                const unsigned long long* root_ptr, char* buf, unsigned cap, int* status) {
-  const char kOp[8] = {'p', '!', '&', '|', 'X', 'F', 'G', 'U'};
-  struct Frame {
-    unsigned long long d;
-    int stage;
-  };
-  Frame st[80];
-  int sp = 0;
-  unsigned n = 0;
-  int bad = 0;
-  st[sp++] = {root_ptr ? *root_ptr : root, 0};
-  auto put = [&](char ch) {
-    if (n + 1 < cap) buf[n++] = ch;
-    else bad = 1;
-  };
-  while (sp > 0 && !bad) {
-    Frame& f = st[sp - 1];
-    const unsigned op = desc_op(f.d);
-    if (op == kAtom) {
-      put('p');
-      char tmp[12];
-      int m = 0;
-      unsigned v = desc_left(f.d);
-      do { tmp[m++] = char('0' + v % 10); v /= 10; } while (v);
-      while (m) put(tmp[--m]);
-      --sp;
-      continue;
-    }
-    const bool bin = op == kAnd || op == kOr || op == kUntil;
-    if (f.stage == 0) {
-      put('(');
-      put(kOp[op & 7]);
-      put(' ');
-      f.stage = 1;
-      if (sp >= 80) { bad = 2; break; }
-      st[sp++] = {prov[desc_left(f.d)], 0};
-    } else if (f.stage == 1 && bin) {
-      put(' ');
-      f.stage = 2;
-      if (sp >= 80) { bad = 2; break; }
-      st[sp++] = {prov[desc_right(f.d)], 0};
-    } else {
-      put(')');
-      --sp;
-    }
-  }
-  buf[n < cap ? n : cap - 1] = '\0';
-  *status = bad;
-}
-
 __global__ void k_reconstruct(const unsigned long long* prov, unsigned long long root,
                               const unsigned long long* root_ptr, char* buf, unsigned cap, int* status) {
-  reconstruct_one(prov, root, root_ptr, buf, cap, status);
+  reconstruct_text(prov, root_ptr ? *root_ptr : root, buf, cap, status);
 }
 
 // One formula per block (thread 0): item i writes buf + i * cap and status[i].
 __global__ void k_reconstruct_many(const lsyn::FormulaItem* items, int n, char* buf, unsigned cap, int* status) {
   const int i = blockIdx.x;
   if (i >= n || threadIdx.x != 0) return;
-  reconstruct_one(items[i].prov, 0, items[i].root, buf + size_t(i) * cap, cap, status + i);
+  reconstruct_text(items[i].prov, *items[i].root, buf + size_t(i) * cap, cap, status + i);
 }
 
 // Candidates built at level k given the sizes of levels 1..k-1 (sizes[i-1]).
@@ -173,12 +124,20 @@ lsyn_status lsyn::ctx_reconstruct(lsyn_ctx* c, const unsigned long long* root_pt
   k_reconstruct<<<1, 1, 0, c->stream>>>(c->prov, 0, root_ptr, c->fbuf, lsyn_ctx::kFormulaCap, c->fstatus);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return c->cuda_fail(e, "reconstruct");
-  e = cudaMemcpyAsync(c->h_fbuf, c->fbuf, lsyn_ctx::kFormulaCap, cudaMemcpyDeviceToHost, c->stream);
+  // most formulas are short: the whole buffer only for those that are not
+  size_t got = 1024;
+  e = cudaMemcpyAsync(c->h_fbuf, c->fbuf, got, cudaMemcpyDeviceToHost, c->stream);
   if (e == cudaSuccess) e = cudaMemcpyAsync(c->h_fstatus, c->fstatus, sizeof(int), cudaMemcpyDeviceToHost, c->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
   if (e != cudaSuccess) return c->cuda_fail(e, "reconstruct copy");
   if (*c->h_fstatus != 0) return c->fail(LSYN_E_STATE, "formula too deep or too long to print");
-  const size_t len = strnlen(c->h_fbuf, lsyn_ctx::kFormulaCap);
+  if (strnlen(c->h_fbuf, got) == got) {
+    got = lsyn_ctx::kFormulaCap;
+    e = cudaMemcpyAsync(c->h_fbuf, c->fbuf, got, cudaMemcpyDeviceToHost, c->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
+    if (e != cudaSuccess) return c->cuda_fail(e, "reconstruct copy");
+  }
+  const size_t len = strnlen(c->h_fbuf, got);
   if (!out || len + 1 > cap) return c->fail(LSYN_E_INVAL, "formula buffer too small");
   memcpy(out, c->h_fbuf, len + 1);
   return LSYN_OK;
@@ -644,11 +603,16 @@ lsyn_status lsyn::ctx_shell(const lsyn_problem* problem, const lsyn_config* conf
   return LSYN_OK;
 }
 
-// A hash table inside a block: its buckets are read with one aligned load each
-// (an allocator of the caller's may align its blocks to less).
-constexpr size_t kBucketBytes = 32;
-static unsigned long long* table_at(void* p) {
-  const uintptr_t a = (reinterpret_cast<uintptr_t>(p) + kBucketBytes - 1) & ~uintptr_t(kBucketBytes - 1);
+// A hash table of n slots: its buckets are read with one aligned load each, and
+// an allocator of the caller's may align its blocks to less.
+static unsigned long long* get_table(Alloc* mem, unsigned long long n) {
+  constexpr uintptr_t kBucketBytes = 32;
+  void* p = mem->get(size_t(n) * 8);
+  if (reinterpret_cast<uintptr_t>(p) & (kBucketBytes - 1)) {
+    mem->give_back(p);
+    p = mem->get(size_t(n) * 8 + kBucketBytes);
+  }
+  const uintptr_t a = (reinterpret_cast<uintptr_t>(p) + kBucketBytes - 1) & ~(kBucketBytes - 1);
   return p ? reinterpret_cast<unsigned long long*>(a) : nullptr;
 }
 
@@ -667,8 +631,9 @@ lsyn_status lsyn::ctx_create(const lsyn_problem* problem, const lsyn_config* con
   cudaError_t e;
   c->arena = static_cast<uint4*>(c->mem.get(size_t(c->max_entries) * M));
   c->prov = static_cast<unsigned long long*>(c->mem.get(size_t(c->max_entries) * 8));
-  c->table = table_at(c->mem.get(size_t(c->table_cap) * 8 + kBucketBytes));
-  c->ctr = static_cast<DevCounters*>(c->mem.get(sizeof(DevCounters)));
+  c->table = get_table(&c->mem, c->table_cap);
+  c->ctr = static_cast<DevCounters*>(c->mem.get(sizeof(DevCounters) + sizeof(SmallState)));
+  c->small = reinterpret_cast<SmallState*>(c->ctr + 1);
   c->consts = static_cast<uint4*>(c->mem.get(size_t(5) * M));
   c->atoms = static_cast<uint4*>(c->mem.get(size_t(c->n_props) * M));
   c->defer[0] = static_cast<unsigned long long*>(c->mem.get(size_t(c->defer_cap) * 8));
@@ -686,7 +651,7 @@ lsyn_status lsyn::ctx_create(const lsyn_problem* problem, const lsyn_config* con
   c->big_table = c->table;
   c->big_cap = c->table_cap;
   if (c->big_cap >= 8 * lsyn_ctx::kFrontSlots) {
-    c->front_table = table_at(c->mem.get(size_t(lsyn_ctx::kFrontSlots) * 8 + kBucketBytes));
+    c->front_table = get_table(&c->mem, lsyn_ctx::kFrontSlots);
     if (!c->front_table) return bail(LSYN_E_NOMEM, "device allocation failed");
     if ((e = cudaStreamCreateWithFlags(&c->side, cudaStreamNonBlocking)) != cudaSuccess)
       return bail(LSYN_E_CUDA, cudaGetErrorString(e));
@@ -707,6 +672,7 @@ lsyn_status lsyn::ctx_create(const lsyn_problem* problem, const lsyn_config* con
   c->events_ready = true;
 
   e = cudaMemcpyAsync(c->consts, consts.data(), consts.size() * 4, cudaMemcpyHostToDevice, c->stream);
+  if (e == cudaSuccess) e = cudaMemsetAsync(c->small, 0, sizeof(SmallState), c->stream);
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(c->atoms, atoms.data(), atoms.size() * 4, cudaMemcpyHostToDevice, c->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);  // host vectors go out of scope
@@ -754,20 +720,200 @@ lsyn_status lsyn_reset(lsyn_ctx* c) {
   c->level_n.assign(1, 0);
   c->levels_done = 0;
   c->last_incomplete = false;
+  if (e == cudaSuccess && c->needs_reset && c->small) {  // a launch may have ended between its steps
+    e = cudaMemsetAsync(c->small, 0, sizeof(SmallState), c->stream);
+    c->small_turn = 0;
+  }
+  if (e != cudaSuccess) return c->cuda_fail(e, "reset");
   c->needs_reset = false;
   c->constructed = 0;
   c->last_sol = ~0ull;
   return LSYN_OK;
 }
 
+}  // extern "C"
+
+namespace {
+
+constexpr unsigned long long kSmallCandidates = 1ull << 17, kSmallBytes = 128ull << 20;
+
+// The parts of a level's algorithmic bytes that its unary and binary operators
+// moved, from their exact counts: operands (in proportion, where a launch
+// stopped at a solution), one table sector per candidate, a compare read per
+// duplicate, CM + provenance + slot per insert.
+void level_bytes(const lsyn_ctx* c, int k, const DevCounters& h, const LevelPlan& lp, lsyn_level_stats* out) {
+  const double M = double(c->vecs) * 16.0;
+  auto launch_bytes = [&](unsigned kind, double operands, double planned) {
+    const double Cl = double(h.built_k[kind]);
+    const double Ul = double(h.inserted_k[kind]);
+    const double done = planned > 0 ? std::min(1.0, Cl / planned) : 1.0;
+    return operands * done + Cl * 32.0 + (Cl - Ul) * M + Ul * (M + 16.0);
+  };
+  const double planned = double(std::max<int64_t>(0, lsyn::level_candidate_count(c, k)));
+  if (lp.plan.n_splits > 0) out->bytes_binary = launch_bytes(kKindBinary, lp.op_bytes_binary, planned - lp.cand_unary);
+  if (lp.uops && lp.u_count) out->bytes_unary = launch_bytes(kKindUnary, lp.op_bytes_unary, lp.cand_unary);
+}
+
+const char* const kErrorText[] = {"", "hash table probe overflow", "hole log overflow",
+                                  "hole fixup found an inconsistent slot", "inconsistent hole log",
+                                  "hash table rebuild overflow", "a wait between blocks ran out"};
+
+lsyn_status check_failed(lsyn_ctx* c, unsigned error) {
+  return c->fail(LSYN_E_STATE, std::string("internal consistency check failed: ") +
+                                   (error < 7 ? kErrorText[error] : "unknown code"));
+}
+
+// Levels of at most this many candidates are built several to a launch
+// (lsyn_small.cuh): beyond, the level's own launches, with three or four blocks
+// per SM instead of two, make up for their overhead.
+unsigned long long small_limit(const lsyn_ctx* c) {
+  const unsigned long long M = (unsigned long long)c->vecs * 16ull;
+  return std::min(kSmallCandidates, kSmallBytes / M);
+}
+
+// Whether level k may be built that way. Not with a time limit (its kernels
+// stop between batches and leave the level incomplete) or a fixed tile (which
+// asks for a particular kernel).
+bool small_level(const lsyn_ctx* c, int k) {
+  if (c->small_off || c->time_limit_ms > 0 || c->tile_rows || k > kSmallLevels) return false;
+  const int64_t cand = lsyn::level_candidate_count(c, k);
+  const unsigned long long start = c->level_start.back() + c->level_n.back();
+  return cand >= 0 && (unsigned long long)cand <= small_limit(c) &&
+         (!c->front_active || double(start) + double(cand) <= double(c->front_cap) * c->table_load);
+}
+
+// Whether lsyn_enumerate_level would take level k at all.
+bool can_build(const lsyn_ctx* c, int k) {
+  return !c->borrowed && !c->needs_reset && !c->last_incomplete && k == c->levels_done + 1 && k <= 64;
+}
+
+// Builds levels k, k + 1, ... up to `last` in one launch, as long as they are
+// small and none holds a solution; out[i] receives the statistics of level
+// k + i, *built how many there are (0: the caller builds level k itself).
+// text (optional): the formula of a solution in the last of them, if it fits the state.
+lsyn_status small_levels(lsyn_ctx* c, int k, int last, lsyn_level_stats* out, int* built, std::string* text) {
+  *built = 0;
+  const double t0 = lsyn::now_ms();
+  last = std::min(last, kSmallLevels);
+  LevelPlan lp;
+  lsyn::ctx_level_plan(c, k, &lp);
+  SmallArgs a;
+  memset(&a, 0, sizeof(a));
+  a.first_level = k;
+  a.last_level = last;
+  const uint32_t m = c->op_mask;
+  a.u_ops = ((m & LSYN_OP_NOT) ? 1u : 0u) | ((m & LSYN_OP_X) ? 2u : 0u) | ((m & LSYN_OP_F) ? 4u : 0u) |
+            ((m & LSYN_OP_G) ? 8u : 0u);
+  a.b_ops = ((m & LSYN_OP_AND) ? 1u : 0u) | ((m & LSYN_OP_OR) ? 2u : 0u) | ((m & LSYN_OP_U) ? 12u : 0u);
+  a.n_props = unsigned(c->n_props);
+  a.call = ++c->small_calls;
+  a.turn = c->small_turn;
+  a.start = lp.start;
+  a.max_candidates = small_limit(c);
+  a.max_total = c->front_active ? (unsigned long long)(double(c->front_cap) * c->table_load) : ~0ull;
+  for (int i = 1; i < k; ++i) {
+    a.level_start[i] = c->level_start[size_t(i)];
+    a.level_n[i] = c->level_n[size_t(i)];
+  }
+  const LaunchCfg lc{c->stream, c->sms};
+  c->level_budget_ns = 0;
+  const CacheView cv = c->view(c->defer[0], &c->ctr->defer_n[0]);
+  cudaError_t e = cudaSuccess;
+  if (!c->small_how.fn)
+    e = c->word_bits == 32 ? SmallKernels<uint32_t>::prepare(cv, c->sms, &c->small_how)
+                           : SmallKernels<uint64_t>::prepare(cv, c->sms, &c->small_how);
+  if (e != cudaSuccess) return c->cuda_fail(e, "small levels");
+  if (c->timing) cudaEventRecord(c->ev[0], c->stream);
+  e = c->word_bits == 32 ? SmallKernels<uint32_t>::run(cv, c->small_how, a, c->small, c->stream)
+                         : SmallKernels<uint64_t>::run(cv, c->small_how, a, c->small, c->stream);
+  if (e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorNotSupported) {
+    cudaGetLastError();  // (not on the devices this is built for) the levels' own launches do
+    c->small_off = true;
+    return LSYN_OK;
+  }
+  if (c->timing) cudaEventRecord(c->ev[1], c->stream);
+  // its state, with the records of the levels, into the pinned counter snapshots
+  static_assert(sizeof(SmallState) <= sizeof(Snap) * lsyn_ctx::kSnaps, "the state fits the snapshots");
+  const size_t bytes = offsetof(SmallState, rec) + sizeof(SmallLevel) * size_t(last - k + 1);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(c->h_snap, c->small, bytes, cudaMemcpyDeviceToHost, c->stream);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
+  if (e != cudaSuccess) return c->cuda_fail(e, "small levels");
+  const SmallState& done = *reinterpret_cast<const SmallState*>(c->h_snap);
+  if (done.call != a.call) {
+    c->needs_reset = true;  // the launch ended in the middle of a level
+    return check_failed(c, 6);
+  }
+  c->small_turn = done.turn;
+  if (text && done.text_status == 0) text->assign(done.text, strnlen(done.text, sizeof(done.text)));
+  const std::vector<SmallLevel> rec(done.rec, done.rec + std::max(0, std::min(done.n_done, last - k + 1)));
+  double others = 0;
+  for (size_t i = 0; i < rec.size(); ++i) {
+    const SmallLevel& r = rec[i];
+    const int kk = k + int(i);
+    if (i) lsyn::ctx_level_plan(c, kk, &lp);
+    if (r.defer_overflow) return c->fail(LSYN_E_STATE, "deferred list overflow: the level is not exact");
+    if (r.error == 1) return c->fail(LSYN_E_STATE, "hash table probe overflow");
+    if (r.unsettled) return c->fail(LSYN_E_STATE, "deferred candidates did not settle");
+    if (r.error) return check_failed(c, r.error);
+    DevCounters h;
+    memset(&h, 0, sizeof(h));
+    for (int q = 0; q < kLaunchKinds; ++q) {
+      h.built_k[q] = r.built_k[q];
+      h.inserted_k[q] = r.inserted_k[q];
+    }
+    h.sol = r.sol;
+    h.solved = r.solved;
+    h.full = r.full;
+    uint32_t total = r.total;
+    if (r.holes) {  // (rare) the last level of the launch: close them as any level's
+      e = c->word_bits == 32
+              ? Kernels<uint32_t>::close_holes(cv, lp.start, c->hole_bits, c->moves, c->move_cap, lc)
+              : Kernels<uint64_t>::close_holes(cv, lp.start, c->hole_bits, c->moves, c->move_cap, lc);
+      if (e == cudaSuccess)
+        e = cudaMemcpyAsync(&c->h_snap[0].c, c->ctr, sizeof(DevCounters), cudaMemcpyDeviceToHost, c->stream);
+      if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
+      if (e != cudaSuccess) return c->cuda_fail(e, "hole fixup kernels");
+      if (c->h_snap[0].c.error) return check_failed(c, c->h_snap[0].c.error);
+      total = std::min(c->h_snap[0].c.n_entries, c->max_entries);
+    }
+    const lsyn_status st = lsyn::ctx_commit_level(c, kk, h, total, r.deferred, lp, &out[i]);
+    if (st != LSYN_OK) return st;
+    level_bytes(c, kk, h, lp, &out[i]);
+    out[i].ms = double(r.ns) * 1e-6;
+    if (i) others += out[i].ms;
+    ++*built;
+  }
+  if (*built) {  // the launch, and what is left of the call's time, count for its first level
+    out[0].launches = 1;
+    out[0].ms = std::max(out[0].ms, lsyn::now_ms() - t0 - others);
+    float ms = 0;
+    if (c->timing && cudaEventElapsedTime(&ms, c->ev[0], c->ev[1]) == cudaSuccess) out[0].kernel_ms[3] = ms;
+  }
+  return LSYN_OK;
+}
+
+}  // namespace
+
+extern "C" {
+
 lsyn_status lsyn_enumerate_level(lsyn_ctx* c, int32_t k, lsyn_level_stats* out) {
   if (!c) return LSYN_E_INVAL;
   if (c->borrowed) return c->fail(LSYN_E_STATE, "a batch or server problem is driven by its owner");
-  if (c->needs_reset) return c->fail(LSYN_E_STATE, "a level was interrupted by the time limit: reset the context");
+  if (c->needs_reset) return c->fail(LSYN_E_STATE, "a level was interrupted (by the time limit): reset the context");
   if (k != c->levels_done + 1) return c->fail(LSYN_E_STATE, "level k must be levels_done + 1");
   if (c->last_incomplete) return c->fail(LSYN_E_STATE, "the previous level is incomplete (cache full or stopped early)");
   if (k > 64) return c->fail(LSYN_E_INVAL, "levels above 64 are not supported");
   cudaSetDevice(c->device);
+  if (small_level(c, k)) {
+    lsyn_level_stats st;
+    int built = 0;
+    const lsyn_status s = small_levels(c, k, k, &st, &built, nullptr);
+    if (s != LSYN_OK) return s;
+    if (built) {
+      if (out) *out = st;
+      return LSYN_OK;
+    }
+  }
   const double t0 = now_ms();
   LaunchCfg lc{c->stream, c->sms};
   int snap = 0, evn = 0;
@@ -823,8 +969,6 @@ lsyn_status lsyn_enumerate_level(lsyn_ctx* c, int32_t k, lsyn_level_stats* out) 
   // (DevCounters::built_k / inserted_k), so the one read of the counters when
   // the level closes gives every launch's share: no copy between launches.
   CacheView cv = c->view(c->defer[0], &c->ctr->defer_n[0]);
-  bool ran_unary = false, ran_binary = false;
-  const double M = double(c->vecs) * 16.0;
   if (k == 1) {
     ev_begin();
     lsyn_status s = launch_desc(c, cv, nullptr, nullptr, 0, unsigned(c->n_props), lc);
@@ -849,7 +993,6 @@ lsyn_status lsyn_enumerate_level(lsyn_ctx* c, int32_t k, lsyn_level_stats* out) 
       ++launches;
       if (e != cudaSuccess) return c->cuda_fail(e, "unary kernel");
       ev_end(0);
-      ran_unary = true;
     }
     if (lp.plan.n_splits > 0) {
       CacheView bv = cv;
@@ -859,7 +1002,6 @@ lsyn_status lsyn_enumerate_level(lsyn_ctx* c, int32_t k, lsyn_level_stats* out) 
       ++launches;
       if (e != cudaSuccess) return c->cuda_fail(e, "binary kernel");
       ev_end(1);
-      ran_binary = true;
     }
   }
   // Close the level without a host round trip in the common case: one pass
@@ -921,32 +1063,13 @@ lsyn_status lsyn_enumerate_level(lsyn_ctx* c, int32_t k, lsyn_level_stats* out) 
     return c->fail(LSYN_E_TIMEOUT, "time limit passed during level " + std::to_string(k) +
                                        ": the level is incomplete; reset the context before using it again");
   }
-  if (h.error) {
-    static const char* const what[] = {"", "hash table probe overflow", "hole log overflow",
-                                       "hole fixup found an inconsistent slot", "inconsistent hole log",
-                                       "hash table rebuild overflow"};
-    return c->fail(LSYN_E_STATE, std::string("internal consistency check failed: ") +
-                                     (h.error < 6 ? what[h.error] : "unknown code"));
-  }
+  if (h.error) return check_failed(c, h.error);
   const uint32_t total = std::min(h.n_entries, c->max_entries);
   lsyn_status st = ctx_commit_level(c, k, c->h_snap[snap - 1].c, total, deferred, lp, out);
   if (st != LSYN_OK) return st;
   if (out) {
     out->launches = launches;
-    // Per launch, from its exact built / inserted counters: operands, one table
-    // sector per candidate, a compare read per duplicate, CM + provenance +
-    // slot per insert.
-    // a launch that stopped at a solution read its operands only in part: in
-    // proportion to the candidates it built
-    auto launch_bytes = [&](unsigned kind, double operands, double planned) {
-      const double Cl = double(h.built_k[kind]);
-      const double Ul = double(h.inserted_k[kind]);
-      const double done = planned > 0 ? std::min(1.0, Cl / planned) : 1.0;
-      return operands * done + Cl * 32.0 + (Cl - Ul) * M + Ul * (M + 16.0);
-    };
-    const double planned = double(level_candidate_count(c, k) > 0 ? level_candidate_count(c, k) : 0);
-    if (ran_binary) out->bytes_binary = launch_bytes(kKindBinary, lp.op_bytes_binary, planned - lp.cand_unary);
-    if (ran_unary) out->bytes_unary = launch_bytes(kKindUnary, lp.op_bytes_unary, lp.cand_unary);
+    level_bytes(c, k, h, lp, out);
     if (c->timing) {
       for (int i = 0; i < evn; ++i) {
         float ms = 0;
@@ -979,14 +1102,32 @@ lsyn_status lsyn_solve(lsyn_ctx* c, int32_t max_size, lsyn_result* out) {
       result = LSYN_E_TIMEOUT;
       break;
     }
-    lsyn_level_stats st;
-    lsyn_status s = lsyn_enumerate_level(c, k, &st);
+    // one level, or as many small ones as one launch builds
+    lsyn_level_stats got[kSmallLevels];
+    int n = 0;
+    lsyn_status s = LSYN_OK;
+    std::string text;
+    if (can_build(c, k) && small_level(c, k)) s = small_levels(c, k, max_size, got, &n, &text);
+    if (s == LSYN_OK && n == 0) {
+      s = lsyn_enumerate_level(c, k, &got[0]);
+      n = s == LSYN_OK ? 1 : 0;
+    }
+    for (int i = 0; i < n; ++i) {
+      out->launches += got[i].launches;
+      if (out->level_stats && k + i <= out->level_stats_cap) out->level_stats[k + i - 1] = got[i];
+    }
     if (s != LSYN_OK) { result = s; break; }
-    out->launches += st.launches;
-    if (out->level_stats && k <= out->level_stats_cap) out->level_stats[k - 1] = st;
+    k += n - 1;
+    const lsyn_level_stats& st = got[n - 1];  // the earlier ones hold no solution and are complete
     if (st.solved) {
-      out->launches += 1;
-      s = ctx_reconstruct(c, &c->ctr->sol, out->formula, out->formula_cap);
+      if (text.empty()) {
+        out->launches += 1;
+        s = ctx_reconstruct(c, &c->ctr->sol, out->formula, out->formula_cap);
+      } else if (!out->formula || text.size() + 1 > out->formula_cap) {
+        s = c->fail(LSYN_E_INVAL, "formula buffer too small");
+      } else {
+        memcpy(out->formula, text.c_str(), text.size() + 1);
+      }
       if (s != LSYN_OK) { result = s; break; }
       out->found = 1;
       out->size = k;

@@ -30,6 +30,15 @@ struct Alloc {
     if (p) owned.push_back(p);
     return p;
   }
+  void give_back(void* p) {
+    for (size_t i = 0; i < owned.size(); ++i)
+      if (owned[i] == p) {
+        owned.erase(owned.begin() + long(i));
+        if (free) free(p, user);
+        else cudaFree(p);
+        return;
+      }
+  }
   void release_all() {
     for (void* p : owned) {
       if (free) free(p, user);
@@ -151,6 +160,10 @@ struct lsyn_ctx {
   unsigned* hole_bits = nullptr;  // [3 x hole_cap + 32] scratch of the device hole plan
   unsigned move_cap = 0;
   unsigned chunk = 1;
+  lsyn::SmallState* small = nullptr;  // several small levels in one launch (behind the counters)
+  bool small_off = false;             // the device refused such a launch
+  uint32_t small_calls = 0, small_turn = 0;
+  lsyn::SmallLaunch small_how;
   char* fbuf = nullptr;
   int* fstatus = nullptr;
   static constexpr unsigned kFormulaCap = 1u << 16;

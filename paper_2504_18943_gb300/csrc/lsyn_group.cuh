@@ -65,6 +65,9 @@ struct GroupWork {
   const unsigned long long* list;      // list mode: descriptors, or NULL for the atoms
   const unsigned int* list_n;
   unsigned int list_cap, atoms;
+  unsigned int list_from;              // list mode: first descriptor
+  unsigned int chunk;                  // ids reserved at a time, at least
+  int settle;                          // 1: goes on after a solution (deferred candidates)
   int warps, batch;                    // warps per group, left rows per item
 };
 
@@ -201,19 +204,23 @@ __host__ __device__ inline size_t group_smem(int mode, unsigned vecs, int warps,
   return (warps > 1 ? size_t(warps) * 4 * batch * 256 : 0) + kGroupCtlBytes + size_t(group_rows(mode, batch)) * vecs * 16;
 }
 
+// The work of one launch, or of one step of a launch that builds several levels
+// (operand rows are copied and compared past L1, so that rows built by the same
+// launch are read as written); `mem` is the block's dynamic shared memory.
 template <typename W, int MODE, bool MP>
-__global__ void __launch_bounds__(256, group_blocks(MP)) k_group(CacheView cv, GroupWork gw,
-                                                  const __grid_constant__ BinaryPlan plan) {
+__device__ __forceinline__ void group_run(const CacheView& cv, const GroupWork& gw, const BinaryPlan& plan,
+                                          unsigned char* mem) {
+  constexpr unsigned kKind = MODE == kGroupUnary ? kKindUnary : MODE == kGroupBinary ? kKindBinary : kKindOther;
   constexpr int NO = MODE == kGroupList ? 1 : 4;   // candidates per row, pair or descriptor
   constexpr int NR = MODE == kGroupUnary ? 1 : 2;  // operand rows of a candidate
   using Ops = ColumnOps<W, MODE, MP>;
-  extern __shared__ __align__(128) unsigned char group_mem[];
   const int warps = gw.warps, T = 32 * warps, B = gw.batch;
   const int planes = MP ? int(cv.planes) : 1;
   const unsigned pv = MP ? cv.plane_vecs : cv.vecs;
   const int gi = int(threadIdx.x) / T, t = int(threadIdx.x) - gi * T, w = t >> 5, lane = t & 31;
   const int per_block = int(blockDim.x) / T;
-  unsigned char* base = group_mem + size_t(gi) * group_smem(MODE, cv.vecs, warps, B);
+  if (gi >= per_block) return;  // threads left over (a block of eight warps, groups of three)
+  unsigned char* base = mem + size_t(gi) * group_smem(MODE, cv.vecs, warps, B);
   unsigned long long* red = reinterpret_cast<unsigned long long*>(base);  // [warps][4 B][32]
   if (warps > 1) base += size_t(warps) * 4 * B * 256;
   GroupCtl* ctl = reinterpret_cast<GroupCtl*>(base);
@@ -230,11 +237,11 @@ __global__ void __launch_bounds__(256, group_blocks(MP)) k_group(CacheView cv, G
   const int my_cols = int((pv - unsigned(t) + unsigned(T) - 1u) / unsigned(T));  // columns t, t + T, ... of a plane (pv >= T)
 
   unsigned long long total = gw.total;
-  if constexpr (MODE == kGroupList) total = gw.list ? min(*gw.list_n, gw.list_cap) : gw.atoms;
+  if constexpr (MODE == kGroupList) total = gw.list ? min(__ldcg(gw.list_n), gw.list_cap) - gw.list_from : gw.atoms;
   const unsigned long long stride = (unsigned long long)gridDim.x * per_block;
   unsigned long long item = (unsigned long long)blockIdx.x * per_block + gi;
   if (MODE == kGroupList && gw.atoms && blockIdx.x == 0 && threadIdx.x == 0)
-    atomicAdd(&cv.ctr->built_k[cv.kind], total);  // deferred candidates were counted when first built
+    atomicAdd(&cv.ctr->built_k[kKind], total);  // deferred candidates were counted when first built
 
   // operands of item i, by warp 0: n consecutive rows a (left), one row b (right)
   auto map_item = [&](unsigned long long i, int x) {
@@ -275,7 +282,7 @@ __global__ void __launch_bounds__(256, group_blocks(MP)) k_group(CacheView cv, G
       a = S.left_start + a0;
       b = S.right_start + r;
     } else {
-      const uint64_t d = gw.list ? gw.list[i] : pack_desc(kAtom, uint32_t(i), 0);
+      const uint64_t d = gw.list ? __ldcg(gw.list + gw.list_from + i) : pack_desc(kAtom, uint32_t(i), 0);
       a = desc_left(d);
       b = desc_right(d);
       op = desc_op(d);
@@ -324,7 +331,7 @@ __global__ void __launch_bounds__(256, group_blocks(MP)) k_group(CacheView cv, G
 
   if (w == 0) {
     map_item(item, 0);
-    if (lane == 0) ctl->stop = stop_requested(cv) ? 1u : 0u;
+    if (lane == 0) ctl->stop = !gw.settle && stop_requested(cv) ? 1u : 0u;
   }
   sync();
   if (item >= total || ctl->stop) return;  // the same for the whole group
@@ -459,7 +466,7 @@ __global__ void __launch_bounds__(256, group_blocks(MP)) k_group(CacheView cv, G
         }
         claimed = __ballot_sync(kFull, state == kClaimed);
         const unsigned n_claim = unsigned(__popc(claimed)), have = ids_end - ids_next;
-        if (n_claim > have && lane == 0) fresh = atomicAdd(&cv.ctr->n_entries, max(cv.chunk, n_claim - have));
+        if (n_claim > have && lane == 0) fresh = atomicAdd(&cv.ctr->n_entries, max(gw.chunk, n_claim - have));
         const uint32_t cm = __ballot_sync(kFull, state == kCompare), tm = __ballot_sync(kFull, state == kTwin);
         const uint32_t wait = __ballot_sync(kFull, state == kWait);
         if (lane < nq) {
@@ -468,7 +475,7 @@ __global__ void __launch_bounds__(256, group_blocks(MP)) k_group(CacheView cv, G
         }
         if (first) map_item(item + stride, 1 - cur);
         if (lane == 0) {
-          if (first) ctl->stop = stop_requested(cv) ? 1u : 0u;
+          if (first) ctl->stop = !gw.settle && stop_requested(cv) ? 1u : 0u;
           ctl->cmp = cm;
           ctl->twin = tm;
           ctl->wait = wait;
@@ -529,7 +536,7 @@ __global__ void __launch_bounds__(256, group_blocks(MP)) k_group(CacheView cv, G
           const unsigned id = rank < have ? ids_next + rank : fresh + (rank - have);
           if (n_claim > have) {
             ids_next = fresh + (n_claim - have);
-            ids_end = fresh + max(cv.chunk, n_claim - have);
+            ids_end = fresh + max(gw.chunk, n_claim - have);
           } else {
             ids_next += n_claim;
           }
@@ -600,20 +607,30 @@ __global__ void __launch_bounds__(256, group_blocks(MP)) k_group(CacheView cv, G
     WarpDedup::flush(pend);
     if (lane == 0) {
       WarpDedup::log_hole(cv, ids_next, ids_end);
-      if (inserted) atomicAdd(&cv.ctr->inserted_k[cv.kind], (unsigned long long)inserted);
-      if (MODE != kGroupList && built) atomicAdd(&cv.ctr->built_k[cv.kind], (unsigned long long)built);
+      if (inserted) atomicAdd(&cv.ctr->inserted_k[kKind], (unsigned long long)inserted);
+      if (MODE != kGroupList && built) atomicAdd(&cv.ctr->built_k[kKind], (unsigned long long)built);
     }
   }
+}
+
+template <typename W, int MODE, bool MP>
+__global__ void __launch_bounds__(256, group_blocks(MP)) k_group(CacheView cv, GroupWork gw,
+                                                                 const __grid_constant__ BinaryPlan plan) {
+  extern __shared__ __align__(128) unsigned char group_mem[];
+  group_run<W, MODE, MP>(cv, gw, plan, group_mem);
 }
 
 // ---------------------------------------------------------------------------
 // Launchers
 // ---------------------------------------------------------------------------
-inline void group_shape(const CacheView& cv, int mode, unsigned long long work, int sms, GroupWork* gw) {
+// resident: warps of the launch that are resident together
+__host__ __device__ inline void group_shape(const CacheView& cv, int mode, unsigned long long work, unsigned resident,
+                                            GroupWork* gw) {
   const int planes = cv.planes <= 1 ? 1 : int(cv.planes);
   const int n = int((planes == 1 ? cv.vecs : cv.plane_vecs) / 32u);  // columns, in warps
+  // groups of w warps resident together (a block holds eight warps)
   auto groups = [&](int w) {
-    return (unsigned long long)sms * group_blocks(planes > 1) * (unsigned(kGroupMaxWarps) / w);
+    return (unsigned long long)(resident / unsigned(kGroupMaxWarps)) * (unsigned(kGroupMaxWarps) / unsigned(w));
   };
   // The largest item that one warp holds with kGroupVecs vectors a thread and
   // that leaves every group a few; wider matrices take one row or pair an item
@@ -624,12 +641,34 @@ inline void group_shape(const CacheView& cv, int mode, unsigned long long work, 
   int batch = mode == kGroupList ? 1 : kGroupMaxBatch;
   while (batch > 1 && (n * planes * group_rows(mode, batch) > kGroupVecs || work < groups(1) * batch * 4)) --batch;
   const int full = (n * planes * group_rows(mode, batch) + kGroupVecs - 1) / kGroupVecs;
-  int warps = std::max(1, std::min({n, kGroupMaxWarps, full}));
+  int warps = n < full ? n : full;
+  warps = warps < 1 ? 1 : warps > kGroupMaxWarps ? kGroupMaxWarps : warps;
   // A launch with too little work to fill half of the GPU's groups: more warps
   // to a candidate, since the chain of one candidate is then what counts.
   while (batch == 1 && warps * 2 <= kGroupMaxWarps && warps * 2 <= n && work * 2 < groups(warps)) warps *= 2;
   gw->warps = warps;
   gw->batch = batch;
+}
+
+// Cuts the splits into items: `batch` rows of the smaller level with one row of
+// the larger; a level with itself in folds of two right-hand rows (n - 1 - r and
+// r) whose items together number the same for every r, or one less.
+__host__ __device__ inline unsigned long long group_items(BinaryPlan* plan, unsigned batch) {
+  unsigned long long total = 0;
+  for (int i = 0; i < plan->n_splits; ++i) {
+    Split& S = plan->s[i];
+    const unsigned rows = S.tri ? S.left_n - 1u : S.left_n;
+    S.lt_tiles = (rows + batch - 1u) / batch + (S.tri ? 1u : 0u);
+    S.rt_tiles = S.tri ? S.left_n / 2u + (S.left_n & 1u) : S.right_n;
+    S.tiles_begin = total;
+    total += (unsigned long long)S.lt_tiles * S.rt_tiles;
+  }
+  plan->total_tiles = total;
+  return total;
+}
+
+inline unsigned group_resident(const CacheView& cv, const LaunchCfg& lc) {
+  return unsigned(lc.sms) * unsigned(group_blocks(cv.planes > 1)) * unsigned(kGroupMaxWarps);
 }
 
 template <typename W, int MODE, bool MP>
@@ -665,7 +704,8 @@ template <typename W>
 cudaError_t GroupKernels<W>::unary(const CacheView& cv, uint32_t first, uint32_t count, uint32_t ops,
                                    const LaunchCfg& lc) {
   GroupWork gw{};
-  group_shape(cv, kGroupUnary, count, lc.sms, &gw);
+  group_shape(cv, kGroupUnary, count, group_resident(cv, lc), &gw);
+  gw.chunk = cv.chunk;
   gw.first = first;
   gw.count = count;
   gw.ops = ops;
@@ -678,26 +718,12 @@ cudaError_t GroupKernels<W>::unary(const CacheView& cv, uint32_t first, uint32_t
 template <typename W>
 cudaError_t GroupKernels<W>::binary(const CacheView& cv, const BinaryPlan& plan, const LaunchCfg& lc) {
   GroupWork gw{};
-  group_shape(cv, kGroupBinary, plan.total_pairs, lc.sms, &gw);
+  group_shape(cv, kGroupBinary, plan.total_pairs, group_resident(cv, lc), &gw);
+  gw.chunk = cv.vecs <= kGroupChunkMaxVecs ? std::min(cv.chunk, kGroupChunk) : 1u;
   gw.ops = plan.ops;
-  // items: `batch` rows of the smaller level with one row of the larger; a
-  // level with itself in folds of two right-hand rows (n - 1 - r and r) whose
-  // items together number the same for every r, or one less
   BinaryPlan items = plan;
-  const unsigned b = unsigned(gw.batch);
-  unsigned long long total = 0;
-  for (int i = 0; i < items.n_splits; ++i) {
-    Split& S = items.s[i];
-    const unsigned rows = S.tri ? S.left_n - 1u : S.left_n;
-    S.lt_tiles = (rows + b - 1u) / b + (S.tri ? 1u : 0u);
-    S.rt_tiles = S.tri ? S.left_n / 2u + (S.left_n & 1u) : S.right_n;
-    S.tiles_begin = total;
-    total += (unsigned long long)S.lt_tiles * S.rt_tiles;
-  }
-  gw.total = items.total_tiles = total;
-  CacheView gv = cv;
-  gv.chunk = cv.vecs <= kGroupChunkMaxVecs ? std::min(cv.chunk, kGroupChunk) : 1u;
-  return group_dispatch<W, kGroupBinary>(gv, gw, items, total, lc);
+  gw.total = group_items(&items, unsigned(gw.batch));
+  return group_dispatch<W, kGroupBinary>(cv, gw, items, gw.total, lc);
 }
 
 template <typename W>
@@ -705,7 +731,8 @@ cudaError_t GroupKernels<W>::desc_list(const CacheView& cv, const unsigned long 
                                        unsigned int cap, unsigned int atoms, const LaunchCfg& lc) {
   GroupWork gw{};
   const unsigned n = list ? cap : atoms;
-  group_shape(cv, kGroupList, n, lc.sms, &gw);
+  group_shape(cv, kGroupList, n, group_resident(cv, lc), &gw);
+  gw.chunk = cv.chunk;
   gw.list = list;
   gw.list_n = list_n;
   gw.list_cap = cap;

@@ -240,4 +240,50 @@ struct GroupKernels {
   static cudaError_t binary(const CacheView& cv, const BinaryPlan& plan, const LaunchCfg& lc);
 };
 
+// Several small levels of one problem in one launch (lsyn_small.cuh).
+constexpr int kSmallLevels = 64;
+
+struct SmallLevel {              // the counters of one level as it closed
+  unsigned long long built_k[kLaunchKinds], inserted_k[kLaunchKinds];
+  unsigned long long sol, ns;    // smallest separating descriptor; time on the GPU
+  unsigned int solved, full, error, defer_overflow;
+  unsigned int unsettled;        // 1: deferred candidates did not settle
+  unsigned int deferred, holes, total;
+};
+
+struct SmallArgs {
+  int first_level, last_level;
+  uint32_t u_ops, b_ops;         // unary and binary operators (LevelPlan, BinaryPlan)
+  uint32_t n_props, start;       // first id of the first level
+  uint32_t list_warps;           // (set by the launcher)
+  uint32_t call, turn;           // names the launch in its state; the state's turn when it starts
+  unsigned long long max_candidates, max_total;  // of a level, and of entries after it at most
+  uint32_t level_start[kSmallLevels + 1], level_n[kSmallLevels + 1];  // of the levels below first_level
+};
+
+struct SmallState {              // in device memory, zeroed once; read back after a launch
+  unsigned int arrived, turn;    // blocks that finished the step; steps begun so far
+  uint32_t call;                 // the launch that n_done and rec belong to
+  int n_done;
+  int text_status;               // 0: `text` is the formula of the last level's solution
+  char text[1024];
+  SmallLevel rec[kSmallLevels];
+  unsigned int words[640];       // the step that the blocks are to take
+};
+
+struct SmallLaunch {             // the launch shape, fixed for a context
+  const void* fn = nullptr;
+  unsigned blocks = 0, list_warps = 0;
+  size_t smem = 0;
+};
+
+template <typename W>
+struct SmallKernels {
+  static cudaError_t prepare(const CacheView& cv, int sms, SmallLaunch* out);
+  // One cooperative launch; st->n_done levels are recorded when it is done (none
+  // if the first one is too large).
+  static cudaError_t run(const CacheView& cv, const SmallLaunch& how, const SmallArgs& args, SmallState* st,
+                         cudaStream_t stream);
+};
+
 }  // namespace lsyn

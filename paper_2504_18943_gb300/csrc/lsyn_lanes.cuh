@@ -40,10 +40,18 @@ struct LanesWork {
   const unsigned long long* list; // list mode: descriptors, or NULL for the atoms
   const unsigned int* list_n;
   unsigned int list_cap, atoms;
+  unsigned int list_from;         // list mode: first descriptor
+  int exact;                      // 1: reserve exactly the ids that the claims need
+  int settle;                     // 1: goes on after a solution (deferred candidates)
 };
 
-template <typename W, int V, int MODE>
-__global__ void __launch_bounds__(256, V >= 4 ? 4 : 2) k_lanes(CacheView cv, LanesWork lw, const __grid_constant__ BinaryPlan plan) {
+// The work of one launch or, with kFresh, of one step of a launch that builds
+// several levels: rows of levels that the same launch built are then read past
+// L1 (nothing orders L1 with the other SMs' writes).
+template <typename W, int V, int MODE, bool kFresh>
+__device__ __forceinline__ void lanes_run(const CacheView& cv, const LanesWork& lw, const BinaryPlan& plan) {
+  constexpr unsigned kKind = MODE == kLanesUnary ? kKindUnary : MODE == kLanesBinary ? kKindBinary : kKindOther;
+  auto read = [](const uint4* p) { return kFresh ? __ldcg(p) : __ldg(p); };
   constexpr int NG = 32 / V;                          // rows, pairs or descriptors per warp batch
   constexpr int NO = MODE == kLanesList ? 1 : 4;      // candidates of each
   constexpr int R = NO == 4 && V < 4 ? 4 / V : 1;     // candidates that a lane probes for
@@ -63,7 +71,7 @@ __global__ void __launch_bounds__(256, V >= 4 ? 4 : 2) k_lanes(CacheView cv, Lan
   }
   __syncthreads();
   unsigned long long total = lw.total;
-  if constexpr (MODE == kLanesList) total = lw.list ? min(*lw.list_n, lw.list_cap) : lw.atoms;
+  if constexpr (MODE == kLanesList) total = lw.list ? min(__ldcg(lw.list_n), lw.list_cap) - lw.list_from : lw.atoms;
   const uint32_t ops = MODE == kLanesList ? 1u : lw.ops & 0xFu;
   const unsigned long long warp = (blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x) >> 5;
   const unsigned long long nwarps = ((unsigned long long)gridDim.x * blockDim.x) >> 5;
@@ -80,7 +88,7 @@ __global__ void __launch_bounds__(256, V >= 4 ? 4 : 2) k_lanes(CacheView cv, Lan
   // almost none are left over (holes, to be closed). Near the end of the arena
   // it reserves exactly its claims, so that no id is kept from another warp.
   const unsigned margin = unsigned(nwarps) * 2u * kLanesAhead;
-  const unsigned ahead_below = cv.max_entries > margin ? cv.max_entries - margin : 0u;
+  const unsigned ahead_below = cv.max_entries > margin && !lw.exact ? cv.max_entries - margin : 0u;
   unsigned batches = total > warp * NG ? unsigned((total - warp * NG - 1) / (nwarps * NG)) : 0u;  // after this one
   unsigned seen = 0xFFFFFFFFu;  // the id counter as this warp last saw it
   bool full = false;  // the arena is full: the specification check only
@@ -114,7 +122,7 @@ __global__ void __launch_bounds__(256, V >= 4 ? 4 : 2) k_lanes(CacheView cv, Lan
     if (!it.valid) return;
     if constexpr (MODE == kLanesUnary) {
       it.a_id = lw.first + uint32_t(i);
-      a = __ldg(row(it.a_id) + l);
+      a = read(row(it.a_id) + l);
     } else if constexpr (MODE == kLanesBinary) {
       int sp = 0;
       while (sp + 1 < plan.n_splits && plan.s[sp + 1].pairs_begin <= i) ++sp;
@@ -122,15 +130,15 @@ __global__ void __launch_bounds__(256, V >= 4 ? 4 : 2) k_lanes(CacheView cv, Lan
       const uint2 ab = split_pair(S, i - S.pairs_begin, false);
       it.a_id = S.left_start + ab.x;
       it.b_id = S.right_start + ab.y;
-      a = __ldg(row(it.a_id) + l);
-      b = __ldg(row(it.b_id) + l);
+      a = read(row(it.a_id) + l);
+      b = read(row(it.b_id) + l);
     } else {
-      const uint64_t d = lw.list ? lw.list[i] : pack_desc(kAtom, uint32_t(i), 0);
+      const uint64_t d = lw.list ? __ldcg(lw.list + lw.list_from + i) : pack_desc(kAtom, uint32_t(i), 0);
       it.op = desc_op(d);
       it.a_id = desc_left(d);
       it.b_id = desc_right(d);
-      a = __ldg((it.op == kAtom ? cv.atoms + size_t(it.a_id) * V : row(it.a_id)) + l);
-      if (it.op == kAnd || it.op == kOr || it.op == kUntil) b = __ldg(row(it.b_id) + l);
+      a = read((it.op == kAtom ? cv.atoms + size_t(it.a_id) * V : row(it.a_id)) + l);
+      if (it.op == kAnd || it.op == kOr || it.op == kUntil) b = read(row(it.b_id) + l);
     }
   };
 
@@ -139,7 +147,7 @@ __global__ void __launch_bounds__(256, V >= 4 ? 4 : 2) k_lanes(CacheView cv, Lan
     // L2 slice, which the id counter's atomics load already); a warp whose own
     // claims found the arena full stops claiming at once.
     if ((iter & 3u) == 0) {
-      if (__any_sync(kFull, lane == 0 && stop_requested(cv))) break;
+      if (__any_sync(kFull, lane == 0 && !lw.settle && stop_requested(cv))) break;
       full = full || __any_sync(kFull, lane == 0 && ld_relaxed_u32(&cv.ctr->full) != 0u);
     }
     Item it;
@@ -396,11 +404,17 @@ __global__ void __launch_bounds__(256, V >= 4 ? 4 : 2) k_lanes(CacheView cv, Lan
   flush();
   if (lane == 0) {
     WarpDedup::log_hole(cv, ids_next, ids_end);
-    if (inserted) atomicAdd(&cv.ctr->inserted_k[cv.kind], (unsigned long long)inserted);
-    if (MODE != kLanesList && built) atomicAdd(&cv.ctr->built_k[cv.kind], (unsigned long long)built);
+    if (inserted) atomicAdd(&cv.ctr->inserted_k[kKind], (unsigned long long)inserted);
+    if (MODE != kLanesList && built) atomicAdd(&cv.ctr->built_k[kKind], (unsigned long long)built);
     if (MODE == kLanesList && lw.atoms && blockIdx.x == 0 && threadIdx.x == 0)
-      atomicAdd(&cv.ctr->built_k[cv.kind], total);  // deferred candidates were counted when first built
+      atomicAdd(&cv.ctr->built_k[kKind], total);  // deferred candidates were counted when first built
   }
+}
+
+template <typename W, int V, int MODE>
+__global__ void __launch_bounds__(256, V >= 4 ? 4 : 2) k_lanes(CacheView cv, LanesWork lw,
+                                                               const __grid_constant__ BinaryPlan plan) {
+  lanes_run<W, V, MODE, false>(cv, lw, plan);
 }
 
 // ---------------------------------------------------------------------------
