@@ -1208,48 +1208,48 @@ lsyn_status lsyn_eval(const lsyn_problem* problem, const char* formula, void* ds
   if (config) cfg = *config;
   if (cfg.device >= 0 && cudaSetDevice(cfg.device) != cudaSuccess) { g_create_error = "bad device"; return LSYN_E_CUDA; }
   cudaStream_t stream = static_cast<cudaStream_t>(cfg.stream);
-  const unsigned plane_vecs = std::max(1u, L.plane_vecs_needed);
-  const unsigned vecs = plane_vecs * unsigned(L.planes);
-  const size_t M = size_t(vecs) * 16;
-  std::vector<uint32_t> consts, atoms;
-  pack_host(problem, L, vecs, plane_vecs, &consts, &atoms);
+  // One block of device memory: the results (first, aligned for both word
+  // types), the caller's atom words, node list and lengths, the scratch rows.
+  const size_t wb = size_t(L.word_bits / 8), row = size_t(L.T) * size_t(L.planes) * wb;
+  auto up = [](size_t x) { return (x + 255) & ~size_t(255); };
+  const size_t at_atoms = up(row), at_nodes = at_atoms + up(row * size_t(problem->n_props));
+  const size_t node_bytes = nodes.size() * sizeof(int4), len_bytes = size_t(L.T) * sizeof(int32_t);
+  const size_t at_scratch = at_nodes + up(node_bytes + len_bytes);
   Alloc mem;
   mem.alloc = cfg.alloc;
   mem.free = cfg.free;
   mem.user = cfg.alloc_user;
-  uint4* d_lm = static_cast<uint4*>(mem.get(M));
-  uint4* d_atoms = static_cast<uint4*>(mem.get(size_t(problem->n_props) * M));
-  int4* d_nodes = static_cast<int4*>(mem.get(nodes.size() * sizeof(int4)));
-  uint4* d_scratch = static_cast<uint4*>(mem.get(nodes.size() * M));
-  uint4* d_out = static_cast<uint4*>(mem.get(M));
-  if (!d_lm || !d_atoms || !d_nodes || !d_scratch || !d_out) {
+  char* d = static_cast<char*>(mem.get(at_scratch + nodes.size() * row));
+  if (!d) {
     mem.release_all();
     g_create_error = "device allocation failed";
     return LSYN_E_NOMEM;
   }
-  std::vector<uint8_t> host_out(M);
-  LaunchCfg lc{stream, 1};
-  cudaError_t e = cudaMemcpyAsync(d_lm, consts.data(), M, cudaMemcpyHostToDevice, stream);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(d_atoms, atoms.data(), atoms.size() * 4, cudaMemcpyHostToDevice, stream);
-  if (e == cudaSuccess)
-    e = cudaMemcpyAsync(d_nodes, nodes.data(), nodes.size() * sizeof(int4), cudaMemcpyHostToDevice, stream);
+  std::vector<char> small(node_bytes + len_bytes);
+  memcpy(small.data(), nodes.data(), node_bytes);
+  memcpy(small.data() + node_bytes, problem->lengths, len_bytes);
+  cudaError_t e = cudaMemcpyAsync(d + at_atoms, problem->atom_words, row * size_t(problem->n_props),
+                                  cudaMemcpyHostToDevice, stream);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(d + at_nodes, small.data(), small.size(), cudaMemcpyHostToDevice, stream);
   if (e == cudaSuccess) {
-    if (L.word_bits == 32)
-      e = Kernels<uint32_t>::eval(d_atoms, d_lm, plane_vecs, unsigned(L.planes), d_nodes, int(nodes.size()), L.steps,
-                                  reinterpret_cast<uint32_t*>(d_scratch), reinterpret_cast<uint32_t*>(d_out), lc);
-    else
-      e = Kernels<uint64_t>::eval(d_atoms, d_lm, plane_vecs, unsigned(L.planes), d_nodes, int(nodes.size()), L.steps,
-                                  reinterpret_cast<uint64_t*>(d_scratch), reinterpret_cast<uint64_t*>(d_out), lc);
+    const int* lengths = reinterpret_cast<const int*>(d + at_nodes + node_bytes);
+    const int4* list = reinterpret_cast<const int4*>(d + at_nodes);
+    auto run = [&](auto w) {
+      using W = decltype(w);
+      return Kernels<W>::eval(reinterpret_cast<const W*>(d + at_atoms), lengths, unsigned(L.T), unsigned(L.planes), list,
+                              int(nodes.size()), L.steps, reinterpret_cast<W*>(d + at_scratch),
+                              reinterpret_cast<W*>(d), stream);
+    };
+    e = L.word_bits == 32 ? run(uint32_t(0)) : run(uint64_t(0));
   }
-  if (e == cudaSuccess) e = cudaMemcpyAsync(host_out.data(), d_out, M, cudaMemcpyDeviceToHost, stream);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(dst, d, row, cudaMemcpyDeviceToHost, stream);
+  const cudaError_t synced = cudaStreamSynchronize(stream);  // also before the host buffers go
+  if (e == cudaSuccess) e = synced;
   mem.release_all();
   if (e != cudaSuccess) {
     g_create_error = std::string("eval: ") + cudaGetErrorString(e);
     return LSYN_E_CUDA;
   }
-  // back to the ABI's [trace][plane] words with bit t = position t
-  planes_to_abi(host_out.data(), static_cast<uint8_t*>(dst), L.T, L.planes, plane_vecs, L.word_bits);
   return LSYN_OK;
 }
 

@@ -215,10 +215,11 @@ struct Kernels {
   // run them; no host round trip. `bits` is scratch of 3 x hole_cap + 32 words.
   static cudaError_t close_holes(const CacheView& cv, unsigned start, unsigned* bits, uint2* moves, unsigned move_cap,
                                  const LaunchCfg& lc);
-  // Evaluate a postorder node list on every trace word of every plane:
-  // scratch [n_nodes][planes][plane words]; a CM of planes x plane_vecs vectors.
-  static cudaError_t eval(const uint4* atoms, const uint4* lenmask, unsigned plane_vecs, unsigned planes,
-                          const int4* nodes, int n_nodes, int steps, W* scratch, W* out, const LaunchCfg& lc);
+  // Evaluate a postorder node list on every trace: atom words [prop][trace]
+  // [plane], lengths and out [trace][plane] in the interface's layout, scratch
+  // [n_nodes][planes][traces].
+  static cudaError_t eval(const W* atoms, const int* lengths, unsigned traces, unsigned planes, const int4* nodes,
+                          int n_nodes, int steps, W* scratch, W* out, cudaStream_t stream);
 };
 
 // Level kernels for CMs of at most 128 bytes (lsyn_lanes.cuh).
