@@ -489,11 +489,7 @@ void lsyn_destroy(lsyn_ctx* c) {
   for (auto& e : c->ev_side) if (e) cudaEventDestroy(e);
   if (c->side) cudaStreamDestroy(c->side);
   c->mem.release_all();
-  if (c->owns_host) {
-    if (c->h_snap) cudaFreeHost(c->h_snap);
-    if (c->h_fbuf) cudaFreeHost(c->h_fbuf);
-    if (c->h_fstatus) cudaFreeHost(c->h_fstatus);
-  }
+  if (c->owns_host) cudaFreeHost(c->h_snap);  // one block, see ctx_create
   if (prev >= 0) cudaSetDevice(prev);
   delete c;
 }
@@ -660,16 +656,21 @@ lsyn_status lsyn::ctx_create(const lsyn_problem* problem, const lsyn_config* con
         return bail(LSYN_E_CUDA, cudaGetErrorString(e));
     c->front_cap = lsyn_ctx::kFrontSlots;
   }
-  if (cudaMallocHost(&c->h_snap, sizeof(Snap) * lsyn_ctx::kSnaps) != cudaSuccess ||
-      cudaMallocHost(&c->h_fbuf, lsyn_ctx::kFormulaCap) != cudaSuccess ||
-      cudaMallocHost(&c->h_fstatus, sizeof(int)) != cudaSuccess) {
+  // one pinned block: the counter snapshots, the formula text and its status
+  // (pinning a block and releasing it are calls into the driver of their own)
+  char* pinned = nullptr;
+  if (cudaMallocHost(&pinned, sizeof(Snap) * lsyn_ctx::kSnaps + lsyn_ctx::kFormulaCap + sizeof(int)) != cudaSuccess) {
     cudaGetLastError();
     return bail(LSYN_E_NOMEM, "pinned host allocation failed");
   }
+  c->h_snap = reinterpret_cast<Snap*>(pinned);
+  c->h_fbuf = pinned + sizeof(Snap) * lsyn_ctx::kSnaps;
+  c->h_fstatus = reinterpret_cast<int*>(c->h_fbuf + lsyn_ctx::kFormulaCap);
   c->owns_host = true;
-  for (auto& ev : c->ev)
-    if ((e = cudaEventCreate(&ev)) != cudaSuccess) return bail(LSYN_E_CUDA, cudaGetErrorString(e));
   c->events_ready = true;
+  if (c->timing)  // the only use of these events
+    for (auto& ev : c->ev)
+      if ((e = cudaEventCreate(&ev)) != cudaSuccess) return bail(LSYN_E_CUDA, cudaGetErrorString(e));
 
   e = cudaMemcpyAsync(c->consts, consts.data(), consts.size() * 4, cudaMemcpyHostToDevice, c->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(c->small, 0, sizeof(SmallState), c->stream);
