@@ -491,8 +491,11 @@ struct PathA {
 
   // Spec check, then probe / compare / insert one candidate.
   // `full`: the arena is full, so only the spec check is done (see path C).
+  // Returns 1 if it was inserted; kMetPending (without `last`) if it met a slot
+  // that another candidate with its hash has claimed and not published.
+  static constexpr unsigned kMetPending = 2;
   __device__ static unsigned process(const CacheView& cv, const Consts& s, const uint4 (&c)[V], uint64_t desc,
-                                     bool full) {
+                                     bool full, bool last) {
     uint32_t lo = 0, hi = 0, bad = 0;
 #pragma unroll
     for (int v = 0; v < V; ++v) {
@@ -508,7 +511,11 @@ struct PathA {
       uint32_t id1;
       const int saw = see_bucket(cv.table, cv.table_mask, pos, tag, id1);
       if (saw == kSeeFull) return 0;
-      if (saw == kSeePending) { defer(cv, desc); return 0; }
+      if (saw == kSeePending) {
+        if (!last) return kMetPending;
+        defer(cv, desc);
+        return 0;
+      }
       if (saw == kSeeMatch) {
         const uint4* src = row_ptr(cv, id1 - 1u);
         uint32_t ne = 0;
@@ -595,6 +602,15 @@ template <> __device__ __forceinline__ uint32_t bit0s<uint32_t>(uint4 c) {
   return (c.x >> 31) | ((c.y >> 31) << 1) | ((c.z >> 31) << 2) | ((c.w >> 31) << 3);
 }
 template <> __device__ __forceinline__ uint32_t bit0s<uint64_t>(uint4 c) { return (c.y >> 31) | ((c.w >> 31) << 1); }
+
+// Probes of a pending slot (a fraction of a microsecond apart) before a warp of
+// the batch kernels defers the candidate. A deferred candidate costs its step
+// another launch and a round trip to the host (50-100 us beside kernels of
+// 150-1800 us). 64 problems of up to 8 KiB a matrix, whole batch: 14.5 ms
+// deferring at once, 14.4 with 16 probes (most steps still deferred some: the
+// owner of a slot writes up to 32 rows before it publishes), 13.6 with 64 (one
+// step of eight did).
+constexpr unsigned kWarpWaits = 64;
 
 // Warp-batch bookkeeping shared by paths C and D: probe states, pending
 // publication of claimed slots, and per-warp id reservations.
@@ -1314,6 +1330,7 @@ struct PathD {
     if (kEarlyPublish) WarpDedup::flush(pend);
     uint32_t cmp_id = 0;
     unsigned long long guard = 0;
+    for (unsigned waits = 0;; ++waits) {  // again for candidates that met a pending slot (below)
     while (true) {
       // Read the buckets; then claims of empty slots and compares, in flight
       // together. A lost claim reads its bucket again in the next round.
@@ -1418,7 +1435,20 @@ struct PathD {
         }
       }
     }
-    if (state == kDeferred) defer(cv, my_desc);
+    // This batch's rows are published at once: warps of other problems' batches
+    // come between this warp's next one, and an equal candidate waits meanwhile.
+    // A pending slot is probed again a few times (the other warp's row is usually
+    // there by then); only then is the candidate deferred, which costs the
+    // step a launch and a round trip to the host.
+    WarpDedup::flush(pend);
+    if (!__any_sync(kFull, state == kDeferred)) break;
+    if (waits >= kWarpWaits) {
+      if (state == kDeferred) defer(cv, my_desc);
+      break;
+    }
+    __nanosleep(200);
+    state = state == kDeferred ? kProbing : kDone;
+    }
   }
 };
 
@@ -1572,11 +1602,11 @@ __device__ __forceinline__ unsigned long long grab(unsigned long long* counter) 
 // The problem's constants sit in this warp's shared slot `ca`, laid out as
 // PathA<W, V>::Consts.
 template <typename W, int V>
-__device__ __forceinline__ unsigned batch_a_one(const CacheView& cv, const uint4* ca, uint64_t d) {
+__device__ __forceinline__ unsigned batch_a_one(const CacheView& cv, const uint4* ca, uint64_t d, bool last) {
   const auto& s = *reinterpret_cast<const typename PathA<W, V>::Consts*>(ca);
   uint4 c[V];
   rebuild_a<W, V>(cv, s, d, c);
-  return PathA<W, V>::process(cv, s, c, d, ld_relaxed_u32(&cv.ctr->full) != 0u);
+  return PathA<W, V>::process(cv, s, c, d, ld_relaxed_u32(&cv.ctr->full) != 0u, last);
 }
 
 template <typename W>
@@ -1594,16 +1624,25 @@ __device__ __forceinline__ void batch_a_load(const CacheView& cv, uint4* ca) {
 // Every lane with `on` set settles descriptor d; returns the warp's inserts.
 template <typename W>
 __device__ unsigned batch_a(const CacheView& cv, const uint4* ca, uint64_t d, bool on) {
-  unsigned ins = 0;
-  if (on) {
-    switch (cv.vecs) {
-      case 1: ins = batch_a_one<W, 1>(cv, ca, d); break;
-      case 2: ins = batch_a_one<W, 2>(cv, ca, d); break;
-      case 4: ins = batch_a_one<W, 4>(cv, ca, d); break;
-      default: ins = batch_a_one<W, 8>(cv, ca, d); break;
+  // a candidate that met a pending slot is tried again, as in the warp paths
+  // (the warp's own claims are published by then)
+  unsigned total = 0;
+  for (unsigned waits = 0; __any_sync(kFull, on); ++waits) {
+    if (waits) __nanosleep(64);
+    unsigned ins = 0;
+    const bool last = waits >= kWarpWaits;
+    if (on) {
+      switch (cv.vecs) {
+        case 1: ins = batch_a_one<W, 1>(cv, ca, d, last); break;
+        case 2: ins = batch_a_one<W, 2>(cv, ca, d, last); break;
+        case 4: ins = batch_a_one<W, 4>(cv, ca, d, last); break;
+        default: ins = batch_a_one<W, 8>(cv, ca, d, last); break;
+      }
     }
+    on = ins == PathA<W, 1>::kMetPending;
+    total += unsigned(__popc(__ballot_sync(kFull, ins == 1u)));
   }
-  return __reduce_add_sync(kFull, ins);
+  return total;
 }
 
 template <typename W, int VPT>

@@ -859,7 +859,6 @@ lsyn_status Engine::answer(const std::vector<Job*>& solved) {
 lsyn_status Engine::run_group(std::vector<Plan>& g, int word_bits, int sms) {
   const int n = int(g.size());
   const unsigned R = rows_per_item();
-  const unsigned long long warps = (unsigned long long)sms * unsigned(tune_.blocks_per_sm) * 8ull;
   // 1. plan every job's level and pack the step array
   unsigned long long tu = 0, tb = 0, td = 0;
   for (int i = 0; i < n; ++i) {
@@ -870,10 +869,10 @@ lsyn_status Engine::run_group(std::vector<Plan>& g, int word_bits, int sms) {
       err = "too many splits for a batch level";
       return LSYN_E_UNSUPPORTED;
     }
-    // Warps move between problems and return their unused ids at each move:
-    // size the id chunk by this job's expected inserts over the launch's warps.
-    const unsigned long long cand = candidates(p.j, p.k);
-    c->chunk = unsigned(std::max(1ull, std::min<unsigned long long>(c->chunk, (cand + 32ull) / (8ull * warps))));
+    // Warps move between problems: they reserve exactly the ids of their claims
+    // (a step's atomics spread over its problems' counters), so that a step
+    // leaves no holes, whose closing would take the host three more round trips.
+    c->chunk = 1;
     StepProblem& sp = h_steps_[i];
     memset(&sp, 0, sizeof(sp));
     sp.cv = c->view(c->defer[0], &c->ctr->defer_n[0]);
