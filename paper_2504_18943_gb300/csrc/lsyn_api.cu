@@ -368,6 +368,17 @@ void lsyn::ctx_level_plan(lsyn_ctx* c, int k, LevelPlan* lp) {
     const long long cand = level_candidate_count(c, k);
     if (cand > 0)
       c->chunk = unsigned(std::max(1ull, std::min<unsigned long long>(c->chunk, (unsigned long long)cand / (8ull * warps))));
+    // Path A (lanes_run) reserves ahead only in a level whose every candidate
+    // would fit beside all that its warps can leave over (two launches, up to 64
+    // warps an SM), so that no id left over can fill the cache, and only with
+    // the log they need. 64-byte matrices, whole level, exact against ahead:
+    // 137 / 146 us at 0.74 M candidates (no holes to close), 245 / 235 at
+    // 2.5 M, 1590 / 1370 at 28 M, where the counter takes one atomic in 1.3 ns.
+    if (c->path == 1) {
+      const unsigned long long over = (unsigned long long)c->sms * 64ull * 2ull * kLanesAhead;
+      c->chunk = cand > (1ll << 20) && (unsigned long long)cand + over <= free_ids && c->hole_cap >= 1u << 16
+                     ? kLanesAhead : 1u;
+    }
   }
   const double M = double(c->vecs) * 16.0;
   if (k == 1) {

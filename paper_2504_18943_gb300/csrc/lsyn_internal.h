@@ -47,6 +47,8 @@ constexpr uint32_t kSlotTomb = 0xFFFFFFFEu;     // claimed, but the arena was fu
 // the batch kernels).
 constexpr int kLaunchKinds = 4;
 constexpr unsigned kKindUnary = 0, kKindBinary = 1, kKindOther = 2;
+// Ids that a warp of a large path-A level reserves beyond its need.
+constexpr unsigned kLanesAhead = 64;
 
 struct alignas(128) DevCounters {
   // ---- the id counter (an atomic per warp chunk) ----
@@ -111,7 +113,7 @@ struct CacheView {
   unsigned int* homes;           // [max_entries]: low 32 bits of each entry's hash (table rebuilds)
   uint2* holes;                  // [hole_cap]: unused id ranges [x, y) left by warps
   unsigned int hole_cap;
-  unsigned int chunk;            // ids a warp reserves per counter update (path B)
+  unsigned int chunk;            // ids a warp reserves per counter update; 1: exactly its claims'
   int steps;                     // log-step count: 2^steps >= longest trace (at most the word width)
   int early_exit;                // 1: stop at the first separating candidate
   unsigned int planes;           // words per trace: plane j holds positions [j w, (j + 1) w) of every trace

@@ -18,9 +18,9 @@
 //
 // Measured against one thread per CM (complete levels, one GB300): 30 traces
 // (120 bytes), four propositions, levels 1-10 in 2.6 ms instead of 5.2, the
-// last level's binary launch 13.1 G candidates/s instead of 4.8; 14 traces (56
-// bytes), the paper's grammar, levels 1-15 in 7.4 ms instead of 8.5: up to 2.5x
-// faster on launches of 10^5 to 10^7 candidates, equal beyond (21 G/s).
+// last level's binary launch 13.2 G candidates/s instead of 4.8; 14 traces (56
+// bytes), the paper's grammar, levels 1-15 in 7.9 ms instead of 8.5: up to 2.5x
+// faster on launches of 10^5 to 10^7 candidates, 21.5 G/s at 28 M.
 #pragma once
 
 #include "lsyn_device.cuh"
@@ -31,9 +31,6 @@ enum : int { kLanesUnary = 0, kLanesBinary = 1, kLanesList = 2 };
 
 // Probes of a pending slot (about a microsecond each) before a candidate is deferred.
 constexpr unsigned kLanesWaits = 8;
-// Ids that a warp reserves beyond its need.
-constexpr unsigned kLanesAhead = 64;
-
 struct LanesWork {
   unsigned long long total;       // rows or pairs (a list reads its own length)
   uint32_t first, ops;            // unary: first row; enabled operators (4 bits)
@@ -41,14 +38,20 @@ struct LanesWork {
   const unsigned int* list_n;
   unsigned int list_cap, atoms;
   unsigned int list_from;         // list mode: first descriptor
-  int exact;                      // 1: reserve exactly the ids that the claims need
+  int exact;                      // 1: reserve exactly the ids that the claims need (as cv.chunk 1)
   int settle;                     // 1: goes on after a solution (deferred candidates)
 };
 
 // The work of one launch or, with kFresh, of one step of a launch that builds
 // several levels: rows of levels that the same launch built are then read past
 // L1 (nothing orders L1 with the other SMs' writes).
-template <typename W, int V, int MODE, bool kFresh>
+//
+// kOps: the operators compiled in (4 bits; lw.ops is a subset of them): all, or
+// those of the paper's grammar (not, X, F; and, U), whose launches then hash,
+// compare and write a quarter less. 64-byte matrices, 92 M candidates of that
+// grammar: 886 + 3690 us (unary + binary) with all four compiled in, 859 + 3455
+// with three. Two operators compiled in were not tried: no grammar here has them.
+template <typename W, int V, int MODE, bool kFresh, unsigned kOps>
 __device__ __forceinline__ void lanes_run(const CacheView& cv, const LanesWork& lw, const BinaryPlan& plan) {
   constexpr unsigned kKind = MODE == kLanesUnary ? kKindUnary : MODE == kLanesBinary ? kKindBinary : kKindOther;
   auto read = [](const uint4* p) { return kFresh ? __ldcg(p) : __ldg(p); };
@@ -73,6 +76,7 @@ __device__ __forceinline__ void lanes_run(const CacheView& cv, const LanesWork& 
   unsigned long long total = lw.total;
   if constexpr (MODE == kLanesList) total = lw.list ? min(__ldcg(lw.list_n), lw.list_cap) - lw.list_from : lw.atoms;
   const uint32_t ops = MODE == kLanesList ? 1u : lw.ops & 0xFu;
+  auto enabled = [](int o) { return MODE == kLanesList || ((kOps >> o) & 1u) != 0u; };
   const unsigned long long warp = (blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x) >> 5;
   const unsigned long long nwarps = ((unsigned long long)gridDim.x * blockDim.x) >> 5;
   constexpr int kProbing = WarpDedup::kProbing, kDone = WarpDedup::kDone, kClaimed = WarpDedup::kClaimed;
@@ -82,15 +86,12 @@ __device__ __forceinline__ void lanes_run(const CacheView& cv, const LanesWork& 
   for (int r = 0; r < R; ++r) pend_pos[r] = pend_tag[r] = pend_id[r] = 0;
   unsigned built = 0, inserted = 0, iter = 0;  // (a warp's share of a level fits 32 bits)
   unsigned ids_next = 0, ids_end = 0;  // ids reserved and not used yet
-  // All warps' reservations meet at one counter. A warp reserves up to
-  // kLanesAhead ids more than the empty slots it has just met, in the same
-  // atomic, beside the claims themselves; fewer towards its last batch, so that
-  // almost none are left over (holes, to be closed). Near the end of the arena
-  // it reserves exactly its claims, so that no id is kept from another warp.
-  const unsigned margin = unsigned(nwarps) * 2u * kLanesAhead;
-  const unsigned ahead_below = cv.max_entries > margin && !lw.exact ? cv.max_entries - margin : 0u;
+  // All warps' reservations meet at one counter. In a large level a warp
+  // reserves up to kLanesAhead ids more than the empty slots it has just met, in
+  // the same atomic, beside the claims themselves; fewer towards its last batch,
+  // so that almost none are left over (holes, to be closed).
+  const bool ahead = cv.chunk > 1u && !lw.exact;
   unsigned batches = total > warp * NG ? unsigned((total - warp * NG - 1) / (nwarps * NG)) : 0u;  // after this one
-  unsigned seen = 0xFFFFFFFFu;  // the id counter as this warp last saw it
   bool full = false;  // the arena is full: the specification check only
 
   // As WarpDedup::flush: the warp barrier orders the other lanes' row stores
@@ -185,6 +186,7 @@ __device__ __forceinline__ void lanes_run(const CacheView& cv, const LanesWork& 
 #pragma unroll
       for (int o = 0; o < NO; ++o) {
         lo[o] = hi[o] = 0;
+        if (!enabled(o)) continue;
         h_acc(c[o], mul, lo[o], hi[o]);
         bad |= (label_miss<W>(c[o], lab) >> 31) << o;
       }
@@ -263,7 +265,7 @@ __device__ __forceinline__ void lanes_run(const CacheView& cv, const LanesWork& 
         if (empty) won[r] = claim_slot(cv.table + pos[r], tag[r]);
         n_empty += unsigned(__popc(__ballot_sync(kFull, empty)));
       }
-      if (n_empty > ids_end - ids_next && seen < ahead_below) {
+      if (ahead && n_empty > ids_end - ids_next) {
         asked = n_empty - (ids_end - ids_next) + min(kLanesAhead, 2u * batches);
         if (lane == 0) fresh = atomicAdd(&cv.ctr->n_entries, asked);
       }
@@ -272,11 +274,13 @@ __device__ __forceinline__ void lanes_run(const CacheView& cv, const LanesWork& 
       uint32_t ne = 0;
 #pragma unroll
       for (int o = 0; o < NO; ++o) {
+        if (!enabled(o)) continue;
         const uint32_t id = from_owner(cmp[NO == 4 && V < 4 ? o % R : 0], o);
         st[o] = id ? __ldcg(row(id - 1u) + l) : c[o];
       }
 #pragma unroll
-      for (int o = 0; o < NO; ++o) ne |= v_ne(st[o], c[o]) ? 1u << o : 0u;
+      for (int o = 0; o < NO; ++o)
+        if (enabled(o)) ne |= v_ne(st[o], c[o]) ? 1u << o : 0u;
 #pragma unroll
       for (int x = V / 2; x > 0; x /= 2) ne |= __shfl_xor_sync(kFull, ne, x);
 #pragma unroll
@@ -300,10 +304,7 @@ __device__ __forceinline__ void lanes_run(const CacheView& cv, const LanesWork& 
           asked = n_claim - have;
           if (lane == 0) fresh = atomicAdd(&cv.ctr->n_entries, asked);
         }
-        if (asked) {
-          fresh = __shfl_sync(kFull, fresh, 0);
-          seen = fresh + asked;
-        }
+        if (asked) fresh = __shfl_sync(kFull, fresh, 0);
         uint32_t id1[R];  // id + 1 of a row to write
         unsigned rank0 = 0;
 #pragma unroll
@@ -333,6 +334,7 @@ __device__ __forceinline__ void lanes_run(const CacheView& cv, const LanesWork& 
         }
 #pragma unroll
         for (int o = 0; o < NO; ++o) {
+          if (!enabled(o)) continue;
           const uint32_t id = from_owner(id1[NO == 4 && V < 4 ? o % R : 0], o);
           if (id) cv.arena[size_t(id - 1u) * V + l] = c[o];
         }
@@ -411,10 +413,10 @@ __device__ __forceinline__ void lanes_run(const CacheView& cv, const LanesWork& 
   }
 }
 
-template <typename W, int V, int MODE>
+template <typename W, int V, int MODE, unsigned kOps>
 __global__ void __launch_bounds__(256, V >= 4 ? 4 : 2) k_lanes(CacheView cv, LanesWork lw,
                                                                const __grid_constant__ BinaryPlan plan) {
-  lanes_run<W, V, MODE, false>(cv, lw, plan);
+  lanes_run<W, V, MODE, false, kOps>(cv, lw, plan);
 }
 
 // ---------------------------------------------------------------------------
@@ -422,14 +424,14 @@ __global__ void __launch_bounds__(256, V >= 4 ? 4 : 2) k_lanes(CacheView cv, Lan
 // ---------------------------------------------------------------------------
 template <typename W, int V>
 struct LaunchA {
-  template <int MODE>
+  template <int MODE, unsigned kOps>
   static cudaError_t run(const CacheView& cv, const LanesWork& lw, const BinaryPlan& plan, unsigned long long n,
                          const LaunchCfg& lc) {
-    static int occ = occupancy_blocks((const void*)k_lanes<W, V, MODE>, 256, 0);
+    static int occ = occupancy_blocks((const void*)k_lanes<W, V, MODE, kOps>, 256, 0);
     constexpr unsigned long long per_block = 8ull * (32 / V);
     const unsigned long long want = (n + per_block - 1) / per_block;
     const unsigned blocks = unsigned(std::max(1ull, std::min(want, (unsigned long long)lc.sms * occ)));
-    k_lanes<W, V, MODE><<<blocks, 256, 0, lc.stream>>>(cv, lw, plan);
+    k_lanes<W, V, MODE, kOps><<<blocks, 256, 0, lc.stream>>>(cv, lw, plan);
     return cudaGetLastError();
   }
   static cudaError_t desc_list(const CacheView& cv, const unsigned long long* list, const unsigned int* list_n,
@@ -439,9 +441,10 @@ struct LaunchA {
     lw.list_n = list_n;
     lw.list_cap = cap;
     lw.atoms = atoms;
+    lw.exact = 1;
     BinaryPlan none;
     none.n_splits = 0;
-    return run<kLanesList>(cv, lw, none, list ? cap : atoms, lc);
+    return run<kLanesList, 15u>(cv, lw, none, list ? cap : atoms, lc);
   }
   static cudaError_t unary(const CacheView& cv, uint32_t first, uint32_t count, uint32_t ops, const LaunchCfg& lc) {
     LanesWork lw{};
@@ -450,13 +453,17 @@ struct LaunchA {
     lw.ops = ops;
     BinaryPlan none;
     none.n_splits = 0;
-    return run<kLanesUnary>(cv, lw, none, count, lc);
+    // bit 3: G
+    return (ops & 8u) == 0u ? run<kLanesUnary, 7u>(cv, lw, none, count, lc)
+                            : run<kLanesUnary, 15u>(cv, lw, none, count, lc);
   }
   static cudaError_t binary(const CacheView& cv, const BinaryPlan& plan, const LaunchCfg& lc) {
     LanesWork lw{};
     lw.total = plan.total_pairs;
     lw.ops = plan.ops;
-    return run<kLanesBinary>(cv, lw, plan, plan.total_pairs, lc);
+    // bit 1: or
+    return (plan.ops & 2u) == 0u ? run<kLanesBinary, 13u>(cv, lw, plan, plan.total_pairs, lc)
+                                 : run<kLanesBinary, 15u>(cv, lw, plan, plan.total_pairs, lc);
   }
 };
 

@@ -251,10 +251,10 @@ __global__ void __launch_bounds__(256, 2) k_small_lanes(CacheView cv, const __gr
       w.total = s.u_count;
       w.first = s.u_first;
       w.ops = a.u_ops;
-      lanes_run<W, V, kLanesUnary, true>(cv, w, s.plan);
+      lanes_run<W, V, kLanesUnary, true, 15u>(cv, w, s.plan);
       w.total = s.b_items;
       w.ops = a.b_ops;
-      lanes_run<W, V, kLanesBinary, true>(cv, w, s.plan);
+      lanes_run<W, V, kLanesBinary, true, 15u>(cv, w, s.plan);
     } else {
       const bool list = s.step == kStepList;
       w.list = list ? cv.defer_out : nullptr;
@@ -263,7 +263,7 @@ __global__ void __launch_bounds__(256, 2) k_small_lanes(CacheView cv, const __gr
       w.list_from = s.list_from;
       w.atoms = list ? 0u : a.n_props;
       w.settle = 1;
-      lanes_run<W, V, kLanesList, true>(cv, w, s.plan);
+      lanes_run<W, V, kLanesList, true, 15u>(cv, w, s.plan);
     }
   }
 }

@@ -70,3 +70,20 @@ def test_arena_of_exactly_the_levels_size(L, traces, bits, row, depth):
             got = [s.level(k) for k in range(1, depth + 1)]
         assert [st.unique for st in got[:-1]] == sizes[:-1]
         assert got[-1].cache_full == full and got[-1].unique == sizes[-1] - full
+
+
+def test_large_level_with_little_room_or_log(L):
+    """A level of millions of candidates, whose warps reserve ids ahead where
+    they can: in an arena of exactly the entries it needs, and with a hole log
+    of one entry, it is complete all the same."""
+    p = L.pack_problem(_problem(2, 14, 6, 24, 32))
+    depth = 11
+    with L.Synthesizer(p, L.torch_config(cache_bytes=4 << 30, full_levels=True)) as s:
+        stats = [s.level(k) for k in range(1, depth + 1)]
+    sizes = [st.unique for st in stats]
+    assert stats[-1].candidates > 1 << 21 and not stats[-1].cache_full
+    for config in (L.make_config(cache_bytes=_bytes_for(sum(sizes), 64), full_levels=True),
+                   L.torch_config(cache_bytes=4 << 30, full_levels=True, hole_cap=1)):
+        with L.Synthesizer(p, config) as s:
+            got = [s.level(k) for k in range(1, depth + 1)]
+        assert [st.unique for st in got] == sizes and not got[-1].cache_full
