@@ -356,28 +356,30 @@ void lsyn::ctx_level_plan(lsyn_ctx* c, int k, LevelPlan* lp) {
   *lp = LevelPlan();
   memset(&lp->plan, 0, sizeof(lp->plan));
   lp->start = c->level_start.back() + c->level_n.back();
-  // Ids a warp reserves at a time: large enough to keep the shared counter
-  // cold, small enough that the reservations of every resident warp stay a
-  // small part of the free arena.
+  // Ids a warp reserves at a time, beyond what its claims need: what it leaves
+  // over is closed as holes after the level, and counts as entries until then.
+  // So none, except
+  // - in path A (lanes_run) in a large level, whose warps' atomics would come
+  //   faster than the counter takes them (one in 1.3 ns): there, up to
+  //   kLanesAhead, if every candidate would fit beside all that the warps can
+  //   leave over (two launches, up to 64 warps an SM), so that no id left over
+  //   can fill the cache, and if the log takes theirs. 64-byte matrices, whole
+  //   level, exact against ahead: 137 / 146 us at 0.74 M candidates (no holes to
+  //   close), 245 / 235 at 2.5 M, 1590 / 1370 at 28 M;
+  // - a few in a large level of path C, where a batch seldom claims fewer: no
+  //   faster than none (6.92 ms at 52 M candidates; 7.12 with 32 at a time), no
+  //   slower but for the close (6 us), and the hole log keeps its use.
   {
     const unsigned long long free_ids = c->max_entries > lp->start ? c->max_entries - lp->start : 0;
-    const unsigned long long warps = (unsigned long long)c->sms * 24ull;
-    c->chunk = unsigned(std::max(1ull, std::min(32ull, free_ids / (8ull * warps))));
-    // a small level: chunks no larger than its candidates spread over the
-    // warps, so that the ids warps leave unused (holes to close) stay few
     const long long cand = level_candidate_count(c, k);
-    if (cand > 0)
-      c->chunk = unsigned(std::max(1ull, std::min<unsigned long long>(c->chunk, (unsigned long long)cand / (8ull * warps))));
-    // Path A (lanes_run) reserves ahead only in a level whose every candidate
-    // would fit beside all that its warps can leave over (two launches, up to 64
-    // warps an SM), so that no id left over can fill the cache, and only with
-    // the log they need. 64-byte matrices, whole level, exact against ahead:
-    // 137 / 146 us at 0.74 M candidates (no holes to close), 245 / 235 at
-    // 2.5 M, 1590 / 1370 at 28 M, where the counter takes one atomic in 1.3 ns.
+    c->chunk = 1;
     if (c->path == 1) {
       const unsigned long long over = (unsigned long long)c->sms * 64ull * 2ull * kLanesAhead;
-      c->chunk = cand > (1ll << 20) && (unsigned long long)cand + over <= free_ids && c->hole_cap >= 1u << 16
-                     ? kLanesAhead : 1u;
+      if (cand > (1ll << 20) && (unsigned long long)cand + over <= free_ids && c->hole_cap >= 1u << 16)
+        c->chunk = kLanesAhead;
+    } else if (c->path == 2) {
+      const unsigned long long warps = (unsigned long long)c->sms * 24ull;
+      if (cand > (1ll << 22)) c->chunk = unsigned(std::max(1ull, std::min(4ull, free_ids / (8ull * warps))));
     }
   }
   const double M = double(c->vecs) * 16.0;
@@ -991,14 +993,6 @@ lsyn_status lsyn_enumerate_level(lsyn_ctx* c, int32_t k, lsyn_level_stats* out) 
     if (lp.uops && lp.u_count) {
       CacheView uv = cv;
       uv.kind = kKindUnary;
-      // CMs above 512 bytes (path D): a unary batch (one row, four candidates)
-      // streams tens of microseconds of rows, so one id reservation per batch
-      // is cheap beside it, while every id a warp leaves unused costs a row
-      // move (2 M bytes) when the level closes: reserve exactly the batch's
-      // inserts (and no prefetched chunk). The binary kernel's shorter
-      // batches keep their chunks: a reservation per batch slowed it more
-      // than its holes cost.
-      if (c->vecs > 32u) uv.chunk = 1;
       ev_begin();
       e = c->word_bits == 32 ? Kernels<uint32_t>::unary(uv, lp.u_first, lp.u_count, lp.uops, lc)
                              : Kernels<uint64_t>::unary(uv, lp.u_first, lp.u_count, lp.uops, lc);
@@ -1028,7 +1022,6 @@ lsyn_status lsyn_enumerate_level(lsyn_ctx* c, int32_t k, lsyn_level_stats* out) 
       return c->cuda_fail(e, "memset");
     CacheView rv = c->view(c->defer[1 - from], &c->ctr->defer_n[1 - from]);
     rv.early_exit = 0;  // a deferred candidate must be settled even after a solution
-    if (c->vecs > 32u) rv.chunk = 1;  // as the unary kernel's (path D)
     ev_begin();
     lsyn_status s = launch_desc(c, rv, c->defer[from], &c->ctr->defer_n[from], n, 0, lc);
     ++launches;
@@ -1037,12 +1030,14 @@ lsyn_status lsyn_enumerate_level(lsyn_ctx* c, int32_t k, lsyn_level_stats* out) 
     return LSYN_OK;
   };
   auto close_holes = [&]() -> lsyn_status {
-    ev_begin();
-    e = c->word_bits == 32 ? Kernels<uint32_t>::close_holes(cv, start, c->hole_bits, c->moves, c->move_cap, lc)
-                           : Kernels<uint64_t>::close_holes(cv, start, c->hole_bits, c->moves, c->move_cap, lc);
-    launches += 3;
-    if (e != cudaSuccess) return c->cuda_fail(e, "hole fixup kernels");
-    ev_end(3);
+    if (c->chunk > 1u) {  // (else no warp had ids left over)
+      ev_begin();
+      e = c->word_bits == 32 ? Kernels<uint32_t>::close_holes(cv, start, c->hole_bits, c->moves, c->move_cap, lc)
+                             : Kernels<uint64_t>::close_holes(cv, start, c->hole_bits, c->moves, c->move_cap, lc);
+      launches += 3;
+      if (e != cudaSuccess) return c->cuda_fail(e, "hole fixup kernels");
+      ev_end(3);
+    }
     if ((e = take_snap()) != cudaSuccess) return c->cuda_fail(e, "snapshot");
     if ((e = cudaStreamSynchronize(c->stream)) != cudaSuccess) return c->cuda_fail(e, "level sync");
     return LSYN_OK;

@@ -618,17 +618,14 @@ struct WarpDedup {
   enum { kProbing = 0, kDone = 1, kClaimed = 2, kDeferred = 3 };
 
   // Ids this warp reserved from the shared counter and has not used yet:
-  // [next, end). Reserving `chunk` ids per counter update keeps the counter
-  // cold; what a warp leaves unused when it exits is logged as a hole and
-  // filled after the level (Kernels::fixup). With full chunks (32 ids) the
-  // next chunk is reserved at the start of a batch whose inserts may need it
-  // (`pre`, in lane 0; `pre_ok` is warp-uniform): an atomic round trip is long
-  // under load, and this one then overlaps the batch's hashing and probing
-  // instead of delaying its inserts.
+  // [next, end); what it leaves unused when it exits is logged as a hole and
+  // filled after the level (Kernels::fixup). A batch reserves what its claims
+  // need, and `chunk` ids at least. Chunks of 32, reserved a batch ahead, cost
+  // more than they saved: the warps left a few hundred thousand ids of a level
+  // over, whose closing took 107 us (none now, 27 where chunk is 4), and the
+  // kernels of 512-byte matrices took 6.89 ms for 52 M candidates against 6.75.
   struct Ids {
     unsigned next = 0, end = 0;
-    unsigned pre = 0;
-    bool pre_ok = false;
     unsigned long long inserted = 0;
     unsigned polls = 0;  // of the arena-full flag
     bool full = false;   // the arena is full
@@ -644,30 +641,12 @@ struct WarpDedup {
     return ids.full;
   }
 
-  __device__ static void prefetch(const CacheView& cv, Ids& ids) {
-    if (!ids.pre_ok && ids.end - ids.next < 32u && cv.chunk >= 32u) {
-      if ((threadIdx.x & 31) == 0) ids.pre = atomicAdd(&cv.ctr->n_entries, cv.chunk);
-      ids.pre_ok = true;
-    }
-  }
-
-  // Ids for a batch's n_claim inserts when the current chunk holds `have`:
-  // the first fresh id (warp-uniform) once the chunk runs out; advances `ids`.
-  // Claim rank r takes ids.next + r while r < have, then fresh + (r - have).
-  __device__ static unsigned take(const Ids& ids, unsigned n_claim, unsigned have, unsigned base, bool use_pre) {
-    return n_claim > have ? __shfl_sync(kFull, use_pre ? ids.pre : base, 0) : 0u;
-  }
-  // Ids reserved on demand for a batch that needs n_claim - have more: a full
-  // chunk, or exactly those in a warp's last batch (nothing is left to hole).
-  __device__ static unsigned demand(const CacheView& cv, unsigned n_claim, unsigned have, bool last) {
-    return last ? n_claim - have : max(cv.chunk, n_claim - have);
-  }
-  __device__ static void advance(const CacheView& cv, Ids& ids, unsigned n_claim, unsigned have, unsigned fresh,
-                                 bool use_pre, bool last = false) {
+  // After a batch of n_claim inserts, of which the warp had ids for `have`:
+  // claim rank r took ids.next + r while r < have, then fresh + (r - have).
+  __device__ static void advance(const CacheView& cv, Ids& ids, unsigned n_claim, unsigned have, unsigned fresh) {
     if (n_claim > have) {
       ids.next = fresh + (n_claim - have);
-      ids.end = fresh + (use_pre ? cv.chunk : demand(cv, n_claim, have, last));
-      if (use_pre) ids.pre_ok = false;
+      ids.end = fresh + max(cv.chunk, n_claim - have);
     } else {
       ids.next += n_claim;
     }
@@ -685,11 +664,9 @@ struct WarpDedup {
     const int lane = threadIdx.x & 31;
     if (lane == 0) {
       log_hole(cv, ids.next, ids.end);
-      if (ids.pre_ok) log_hole(cv, ids.pre, ids.pre + cv.chunk);
       if (ids.inserted) atomicAdd(&cv.ctr->inserted_k[cv.kind], ids.inserted);
     }
     ids.next = ids.end = 0;
-    ids.pre_ok = false;
     ids.inserted = 0;
     ids.polls = 0;
     ids.full = false;
@@ -769,14 +746,10 @@ struct PathC {
   // generators whose consecutive batches share an operand, so that a warp never
   // defers on its own inserts); otherwise after probing, when the fence no
   // longer waits for those stores.
-  // last (warp-uniform): the warp's final batch of the launch; it reserves no
-  // chunk ahead and takes exactly the ids its inserts need, so that its
-  // unused ids (holes, moved at the level's close) stay few.
   template <bool kEarlyPublish, class Gen>
   __device__ static void batch(const CacheView& cv, const Consts& k, const Gen& gen, int n, uint32_t en,
-                               uint4* stage, Pending& pend, Ids& ids, bool last = false) {
+                               uint4* stage, Pending& pend, Ids& ids) {
     const int lane = threadIdx.x & 31;
-    if (!last) WarpDedup::prefetch(cv, ids);
     uint32_t my_lo = 0, my_hi = 0, bad = 0;
     for (int q0 = 0; q0 < n; q0 += 4) {  // n is a multiple of 4: four operators per operand group
       uint4 c4[4];
@@ -881,13 +854,11 @@ struct PathC {
     const uint32_t claim = __ballot_sync(kFull, state == kClaimed);
     const unsigned n_claim = unsigned(__popc(claim));
     const unsigned have = ids.end - ids.next;  // warp-uniform
-    const bool use_pre = n_claim > have && ids.pre_ok;
-    unsigned base = 0;
-    if (n_claim > have && !use_pre && lane == 0)
-      base = atomicAdd(&cv.ctr->n_entries, WarpDedup::demand(cv, n_claim, have, last));
+    unsigned fresh = 0;
+    if (n_claim > have && lane == 0) fresh = atomicAdd(&cv.ctr->n_entries, max(cv.chunk, n_claim - have));
     if (!kEarlyPublish) WarpDedup::flush(pend);  // overlaps the id reservation above
     if (claim) {
-      const unsigned fresh = WarpDedup::take(ids, n_claim, have, base, use_pre);
+      fresh = __shfl_sync(kFull, fresh, 0);
       unsigned rank = 0;
       for (uint32_t m = claim; m; m &= m - 1u, ++rank) {
         const int q = __ffs(m) - 1;
@@ -896,7 +867,7 @@ struct PathC {
       }
       const unsigned my_rank = unsigned(__popc(claim & ((1u << lane) - 1u)));
       const unsigned my_id = my_rank < have ? ids.next + my_rank : fresh + (my_rank - have);
-      WarpDedup::advance(cv, ids, n_claim, have, fresh, use_pre, last);
+      WarpDedup::advance(cv, ids, n_claim, have, fresh);
       const unsigned wrote = unsigned(__popc(__ballot_sync(kFull, state == kClaimed && my_id < cv.max_entries)));
       ids.inserted += wrote;
       ids.full = ids.full || wrote < n_claim;
@@ -1038,8 +1009,7 @@ __global__ void __launch_bounds__(256, 3) k_unary_c(CacheView cv, uint32_t first
     __syncwarp();
     gen.id0 = first + base;
     const uint32_t en = en_ops & ((nrows >= 8u ? 0xFFFFFFFFu : ((1u << (4 * nrows)) - 1u)));
-    const bool last = base + nwarps * ROWS >= count;
-    P::template batch<false>(cv, k, gen, int(4 * nrows), en, stage, pend, idr, last);
+    P::template batch<false>(cv, k, gen, int(4 * nrows), en, stage, pend, idr);
     built += __popc(en);
     __syncwarp();
   }
@@ -1177,11 +1147,10 @@ __global__ void __launch_bounds__(256, 3) k_binary_small_c(CacheView cv, BinaryP
     __syncwarp();
     gen.a0 = S.left_start + l0;
     const uint32_t en = en_ops & (np >= 8u ? 0xFFFFFFFFu : ((1u << (4 * np)) - 1u));
-    const bool last_item = c + nwarps >= plan.total_tiles;
     for (uint32_t r = r0; r < r1; ++r) {
       gen.b_id = S.right_start + r;
       gen.b = __ldg(row_ptr(cv, gen.b_id) + lane);
-      P::template batch<true>(cv, k, gen, int(4 * np), en, stage, pend, idr, last_item && r + 1u == r1);
+      P::template batch<true>(cv, k, gen, int(4 * np), en, stage, pend, idr);
       built += __popc(en);
     }
     __syncwarp();
@@ -1267,7 +1236,6 @@ struct PathD {
 
   template <bool kEarlyPublish, class Gen>
   __device__ static void batch(const CacheView& cv, const Gen& gen, int n, uint32_t en, Pending& pend, Ids& ids) {
-    WarpDedup::prefetch(cv, ids);
     const int lane = threadIdx.x & 31;
     const unsigned rv = cv.vecs >> 5;
     uint32_t my_lo = 0, my_hi = 0, bad = 0;
@@ -1386,13 +1354,11 @@ struct PathD {
     const uint32_t claim = __ballot_sync(kFull, state == kClaimed);
     const unsigned n_claim = unsigned(__popc(claim));
     const unsigned have = ids.end - ids.next;
-    const bool use_pre = n_claim > have && ids.pre_ok;
-    unsigned base = 0;
-    if (n_claim > have && !use_pre && lane == 0)
-      base = atomicAdd(&cv.ctr->n_entries, max(cv.chunk, n_claim - have));
+    unsigned fresh = 0;
+    if (n_claim > have && lane == 0) fresh = atomicAdd(&cv.ctr->n_entries, max(cv.chunk, n_claim - have));
     if (!kEarlyPublish) WarpDedup::flush(pend);
     if (claim) {
-      const unsigned fresh = WarpDedup::take(ids, n_claim, have, base, use_pre);
+      fresh = __shfl_sync(kFull, fresh, 0);
       // the rows of one operand group's claims in one pass over its vectors
       for (uint32_t gm = claim; gm;) {
         const int g = (__ffs(gm) - 1) >> 2;
@@ -1417,7 +1383,7 @@ struct PathD {
       }
       const unsigned my_rank = unsigned(__popc(claim & ((1u << lane) - 1u)));
       const unsigned my_id = my_rank < have ? ids.next + my_rank : fresh + (my_rank - have);
-      WarpDedup::advance(cv, ids, n_claim, have, fresh, use_pre);
+      WarpDedup::advance(cv, ids, n_claim, have, fresh);
       const unsigned wrote = unsigned(__popc(__ballot_sync(kFull, state == kClaimed && my_id < cv.max_entries)));
       ids.inserted += wrote;
       ids.full = ids.full || wrote < n_claim;
@@ -1598,7 +1564,7 @@ __device__ __forceinline__ unsigned long long grab(unsigned long long* counter) 
 
 // Path A inside the batch runner (CMs of at most 8 vectors): every lane holds
 // one candidate, named by its descriptor, rebuilds it from its operands and
-// probes / inserts it alone, exactly as k_unary_a / k_binary_a / k_desc_a do.
+// probes / inserts it alone.
 // The problem's constants sit in this warp's shared slot `ca`, laid out as
 // PathA<W, V>::Consts.
 template <typename W, int V>

@@ -48,10 +48,6 @@ constexpr int kGroupMaxWarps = 8;  // warps that share a candidate (a block)
 constexpr int kGroupVecs = 16;
 constexpr int kGroupMaxBatch = 4;  // left rows per item
 constexpr unsigned kGroupWaits = 12;   // probes of a pending slot (a round trip and two barriers each) before deferring
-// Ids a group of the binary kernel reserves at a time on small matrices (at
-// most 2 KiB): the id counter is then bumped by every second item or so; what
-// is left over when the launch ends costs row moves, so it stays small.
-constexpr unsigned kGroupChunk = 8, kGroupChunkMaxVecs = 128;
 
 // Blocks per SM that the compiler is to leave registers for: three (80
 // registers) fit the one-plane kernels without spills, and four cost 15-25 % in
@@ -66,7 +62,6 @@ struct GroupWork {
   const unsigned int* list_n;
   unsigned int list_cap, atoms;
   unsigned int list_from;              // list mode: first descriptor
-  unsigned int chunk;                  // ids reserved at a time, at least
   int settle;                          // 1: goes on after a solution (deferred candidates)
   int warps, batch;                    // warps per group, left rows per item
 };
@@ -343,7 +338,7 @@ __device__ __forceinline__ void group_run(const CacheView& cv, const GroupWork& 
   constexpr int kProbing = WarpDedup::kProbing, kDone = WarpDedup::kDone, kClaimed = WarpDedup::kClaimed;
   constexpr int kCompare = 4, kWait = 5, kTwin = 6;
   WarpDedup::Pending pend;
-  unsigned ids_next = 0, ids_end = 0, built = 0, inserted = 0;  // (a warp's share of a level fits 32 bits)
+  unsigned built = 0, inserted = 0;  // (a warp's share of a level fits 32 bits)
 
   while (true) {
     const int n = int(uniform(ctl->n[cur]));
@@ -465,8 +460,9 @@ __device__ __forceinline__ void group_run(const CacheView& cv, const GroupWork& 
           }
         }
         claimed = __ballot_sync(kFull, state == kClaimed);
-        const unsigned n_claim = unsigned(__popc(claimed)), have = ids_end - ids_next;
-        if (n_claim > have && lane == 0) fresh = atomicAdd(&cv.ctr->n_entries, max(gw.chunk, n_claim - have));
+        // ids for the claims, exactly as many: a level has no holes to close
+        // (8 at a time on matrices up to 2 KiB measured the same)
+        if (claimed && lane == 0) fresh = atomicAdd(&cv.ctr->n_entries, unsigned(__popc(claimed)));
         const uint32_t cm = __ballot_sync(kFull, state == kCompare), tm = __ballot_sync(kFull, state == kTwin);
         const uint32_t wait = __ballot_sync(kFull, state == kWait);
         if (lane < nq) {
@@ -530,16 +526,7 @@ __device__ __forceinline__ void group_run(const CacheView& cv, const GroupWork& 
       if (w == 0) {  // ids for the claims
         uint32_t wrote = 0;
         if (claimed) {
-          const unsigned n_claim = unsigned(__popc(claimed)), have = ids_end - ids_next;
-          fresh = __shfl_sync(kFull, fresh, 0);
-          const unsigned rank = unsigned(__popc(claimed & ((1u << lane) - 1u)));
-          const unsigned id = rank < have ? ids_next + rank : fresh + (rank - have);
-          if (n_claim > have) {
-            ids_next = fresh + (n_claim - have);
-            ids_end = fresh + max(gw.chunk, n_claim - have);
-          } else {
-            ids_next += n_claim;
-          }
+          const unsigned id = __shfl_sync(kFull, fresh, 0) + unsigned(__popc(claimed & ((1u << lane) - 1u)));
           const bool ok = state == kClaimed && id < cv.max_entries;
           if (state == kClaimed) {
             unsigned long long* slot = cv.table + pos;
@@ -606,7 +593,6 @@ __device__ __forceinline__ void group_run(const CacheView& cv, const GroupWork& 
   if (w == 0) {
     WarpDedup::flush(pend);
     if (lane == 0) {
-      WarpDedup::log_hole(cv, ids_next, ids_end);
       if (inserted) atomicAdd(&cv.ctr->inserted_k[kKind], (unsigned long long)inserted);
       if (MODE != kGroupList && built) atomicAdd(&cv.ctr->built_k[kKind], (unsigned long long)built);
     }
@@ -705,7 +691,6 @@ cudaError_t GroupKernels<W>::unary(const CacheView& cv, uint32_t first, uint32_t
                                    const LaunchCfg& lc) {
   GroupWork gw{};
   group_shape(cv, kGroupUnary, count, group_resident(cv, lc), &gw);
-  gw.chunk = cv.chunk;
   gw.first = first;
   gw.count = count;
   gw.ops = ops;
@@ -719,7 +704,6 @@ template <typename W>
 cudaError_t GroupKernels<W>::binary(const CacheView& cv, const BinaryPlan& plan, const LaunchCfg& lc) {
   GroupWork gw{};
   group_shape(cv, kGroupBinary, plan.total_pairs, group_resident(cv, lc), &gw);
-  gw.chunk = cv.vecs <= kGroupChunkMaxVecs ? std::min(cv.chunk, kGroupChunk) : 1u;
   gw.ops = plan.ops;
   BinaryPlan items = plan;
   gw.total = group_items(&items, unsigned(gw.batch));
@@ -732,7 +716,6 @@ cudaError_t GroupKernels<W>::desc_list(const CacheView& cv, const unsigned long 
   GroupWork gw{};
   const unsigned n = list ? cap : atoms;
   group_shape(cv, kGroupList, n, group_resident(cv, lc), &gw);
-  gw.chunk = cv.chunk;
   gw.list = list;
   gw.list_n = list_n;
   gw.list_cap = cap;

@@ -51,7 +51,7 @@ constexpr unsigned kKindUnary = 0, kKindBinary = 1, kKindOther = 2;
 constexpr unsigned kLanesAhead = 64;
 
 struct alignas(128) DevCounters {
-  // ---- the id counter (an atomic per warp chunk) ----
+  // ---- the id counter (an atomic per warp batch with claims) ----
   unsigned int n_entries;        // arena fill (may exceed max_entries when full)
   unsigned int pad0[31];
   // ---- flags polled by every warp, written rarely ----

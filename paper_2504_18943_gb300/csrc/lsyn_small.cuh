@@ -279,7 +279,6 @@ __global__ void __launch_bounds__(256, 2) k_small_group(CacheView cv, const __gr
     if (!small_next<true>(cv, a, st, &own, &s, turn, begin)) return;
     if (s.step == kStepStop) return;
     GroupWork w{};
-    w.chunk = 1;
     if (s.step == kStepLevel && s.k > 1) {
       if (s.u_count) {
         w.warps = int(s.u_warps);
