@@ -335,7 +335,8 @@ typedef struct {
   int32_t light_sms;      /* SMs the batch steps keep while a large level runs (0 = 1/8 of the SMs) */
   int32_t lanes;          /* large levels of different problems in flight at once (0 = 4) */
   int32_t rows_per_item;  /* formulas per warp: rows of the unary work and pairs of the binary work in
-                             one work item of a batch step, each with its 4 operators (2, 4 or 8; 0 = 8) */
+                             one work item of a batch step, each with its 4 operators (2, 4 or 8; 0 = 8);
+                             a step too small to give every warp two items takes fewer */
   int32_t words_per_thread; /* CMs above 128 bytes: 16-byte vectors a lane loads together in each step
                              of its loops over a CM (1 or 2; 0 = 1) */
   int32_t table_load_pct; /* load, in percent (25..90), up to which a problem's hash table fills before

@@ -1622,7 +1622,7 @@ __global__ void __launch_bounds__(256) k_batch_run(StepHeader* hdr, const StepPr
   CacheView* cv = &s_cv[wib];
   uint4* ca = s_ca[wib];
   const int n = hdr->n;
-  const uint32_t R = uint32_t(hdr->rows);  // unary rows / binary pairs per work item (2, 4 or 8)
+  const uint32_t R = uint32_t(hdr->rows);  // unary rows / binary pairs per work item (1, 2, 4 or 8)
   BatchWarp<W> bw;
   auto enter = [&](int p) {
     const bool fresh = p != bw.cur;

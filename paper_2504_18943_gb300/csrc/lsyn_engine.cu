@@ -858,17 +858,20 @@ lsyn_status Engine::answer(const std::vector<Job*>& solved) {
 
 lsyn_status Engine::run_group(std::vector<Plan>& g, int word_bits, int sms) {
   const int n = int(g.size());
-  const unsigned R = rows_per_item();
   // 1. plan every job's level and pack the step array
-  unsigned long long tu = 0, tb = 0, td = 0;
-  for (int i = 0; i < n; ++i) {
-    Plan& p = g[size_t(i)];
-    lsyn_ctx* c = p.j->c;
-    ctx_level_plan(c, p.k, &p.lp);
+  unsigned long long units = 0, tu = 0, tb = 0, td = 0;  // units: rows and pairs
+  for (Plan& p : g) {
+    ctx_level_plan(p.j->c, p.k, &p.lp);
     if (p.lp.plan.n_splits > kBatchSplits) {
       err = "too many splits for a batch level";
       return LSYN_E_UNSUPPORTED;
     }
+    units += p.lp.u_count + p.lp.plan.total_pairs;
+  }
+  const unsigned R = rows_per_item(units, sms);
+  for (int i = 0; i < n; ++i) {
+    Plan& p = g[size_t(i)];
+    lsyn_ctx* c = p.j->c;
     // Warps move between problems: they reserve exactly the ids of their claims
     // (a step's atomics spread over its problems' counters), so that a step
     // leaves no holes, whose closing would take the host three more round trips.

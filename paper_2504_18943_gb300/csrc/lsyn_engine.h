@@ -233,7 +233,19 @@ class Engine {
   unsigned long long candidates(const Job* j, int k) const;
   unsigned long long solo_min() const { return tune_.solo_candidates ? tune_.solo_candidates : (1ull << 19); }
   // unary rows / binary pairs per work item of a batch step
-  unsigned rows_per_item() const { return tune_.rows_per_item > 0 ? unsigned(tune_.rows_per_item) : 8u; }
+  // Rows or pairs per work item of a step with that many: the tuned number, or
+  // 8, but fewer where the step's resident warps (16 per SM: k_batch_run needs
+  // 128 registers) would otherwise get less than two items each. A warp settles
+  // an item's candidates one batch at a time, so in a small step its chain of
+  // round trips is all that counts. Steps of 10^3 to 3 x 10^4 candidates: 43-90 us
+  // instead of 82-164; a burst of 24 problems on the server 6.51 -> 6.17 ms, a
+  // batch of 64, most of whose time goes to larger steps, within noise (13.1 ->
+  // 12.7). One item a warp gave half of that, four no more than two.
+  unsigned rows_per_item(unsigned long long units, int sms) const {
+    unsigned r = tune_.rows_per_item > 0 ? unsigned(tune_.rows_per_item) : 8u;
+    while (r > 1u && units < (unsigned long long)sms * 32ull * r) r /= 2u;
+    return r;
+  }
   // load up to which a job's table fills before it is rebuilt larger (its entry limit does not depend on it)
   double table_load(const Job* j) const {
     return tune_.table_load_pct > 0 ? double(tune_.table_load_pct) / 100.0 : j->c->table_load;

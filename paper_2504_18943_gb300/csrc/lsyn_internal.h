@@ -169,7 +169,7 @@ struct StepProblem {
 struct alignas(128) StepHeader {
   unsigned long long total_u, total_b, total_d;
   int n;                       // problems in this step
-  int rows;                    // unary rows / binary pairs per work item (2, 4 or 8)
+  int rows;                    // unary rows / binary pairs per work item (1, 2, 4 or 8)
   int pad0[24];
   struct alignas(128) Counter {
     unsigned long long v;

@@ -225,3 +225,20 @@ def test_large_level_lane_matches_plain(L, problems):
                 st, res, f, _ = s.solve(9)
                 for k in _complete_levels(st, res):
                     assert np.array_equal(canon(b.export(i, k)), canon(s.export(k))), (i, k)
+
+
+@pytest.mark.parametrize("n", [1, 3, 40])
+def test_small_and_large_steps_build_the_same_levels(L, n):
+    """A step too small for every warp takes fewer rows a work item (one for a
+    single problem's first levels, eight for many problems' later ones): every
+    problem's complete levels are those of its own context."""
+    packed = [L.pack_problem(W.batched_problem(4000, i, oracle.labeller)) for i in range(n)]
+    cfg = L.make_config(cache_bytes=256 << 20)
+    with L.Batch(packed, cfg) as b:
+        statuses, results, _ = b.solve(7)
+        for i, p in enumerate(packed):
+            with L.Synthesizer(p, cfg) as s:
+                st, res, _, _ = s.solve(7)
+                assert (statuses[i], results[i].size) == (st, res.size), i
+                for k in _complete_levels(st, res):
+                    assert np.array_equal(canon(b.export(i, k)), canon(s.export(k))), (i, k)
