@@ -202,8 +202,8 @@ def _one_problem_workloads():
                                "binary": "k_group (and/or/U level kernel, 16 KiB CMs)"}),
         "e3": dict(make=lambda W, lab, seed: _paper_example(W), cache=16 << 30, max_size=16,
                    op_mask=0x1B | 0x40, dtype="u32", desc=E3_WORKLOAD, steps=5, cpu_levels=(12, 14),
-                   kernels={"unary": "k_unary_a (not/X/F/G level kernel, 64-byte CMs)",
-                            "binary": "k_binary_a (and/U level kernel, 64-byte CMs)"}),
+                   kernels={"unary": "k_lanes (not/X/F/G level kernel, 64-byte CMs)",
+                            "binary": "k_lanes (and/U level kernel, 64-byte CMs)"}),
     }
 
 
@@ -668,7 +668,7 @@ def run_served(args):
 def _kernel_sha() -> str:
     import hashlib
     h = hashlib.sha256()
-    for name in ("lsyn_device.cuh", "lsyn_api.cu", "lsyn_internal.h"):
+    for name in ("lsyn_device.cuh", "lsyn_group.cuh", "lsyn_lanes.cuh", "lsyn_api.cu", "lsyn_internal.h"):
         with open(os.path.join(ROOT, "paper_2504_18943_gb300", "csrc", name), "rb") as f:
             h.update(f.read())
     return h.hexdigest()[:16]

@@ -248,13 +248,12 @@ lsyn_status validate(const lsyn_problem* p, Layout* L, std::string* err) {
 void pack_host(const lsyn_problem* p, const Layout& L, unsigned vecs, unsigned plane_vecs,
                std::vector<uint32_t>* consts, std::vector<uint32_t>* atoms) {
   const unsigned n32 = vecs * 4;  // 32-bit words per padded CM
-  consts->assign(size_t(5) * n32, 0u);
+  consts->assign(size_t(4) * n32, 0u);
   atoms->assign(size_t(p->n_props) * n32, 0u);
   uint32_t* lm = consts->data();
   uint32_t* lab = lm + n32;
   uint32_t* care = lab + n32;
-  uint32_t* key = care + n32;
-  uint32_t* mul = key + n32;
+  uint32_t* mul = care + n32;
   const int per = p->word_bits / 32;  // 32-bit halves per word
   // Words are stored position 0 first (most significant bit); the 32-bit
   // halves of a 64-bit word are little-endian in memory.
@@ -288,10 +287,7 @@ void pack_host(const lsyn_problem* p, const Layout& L, unsigned vecs, unsigned p
       }
     }
   }
-  for (unsigned i = 0; i < n32; ++i) {
-    key[i] = mix32(i * 2u + 0x51ED270Bu);
-    mul[i] = mix32(i * 2u + 0x2545F491u) | 1u;
-  }
+  for (unsigned i = 0; i < n32; ++i) mul[i] = mix32(i * 2u + 0x2545F491u) | 1u;
 }
 
 // One internal row (planes x plane_vecs vectors, position 0 in the top bit)
@@ -643,7 +639,7 @@ lsyn_status lsyn::ctx_create(const lsyn_problem* problem, const lsyn_config* con
   c->table = get_table(&c->mem, c->table_cap);
   c->ctr = static_cast<DevCounters*>(c->mem.get(sizeof(DevCounters) + sizeof(SmallState)));
   c->small = reinterpret_cast<SmallState*>(c->ctr + 1);
-  c->consts = static_cast<uint4*>(c->mem.get(size_t(5) * M));
+  c->consts = static_cast<uint4*>(c->mem.get(size_t(4) * M));
   c->atoms = static_cast<uint4*>(c->mem.get(size_t(c->n_props) * M));
   c->defer[0] = static_cast<unsigned long long*>(c->mem.get(size_t(c->defer_cap) * 8));
   c->defer[1] = static_cast<unsigned long long*>(c->mem.get(size_t(c->defer_cap) * 8));

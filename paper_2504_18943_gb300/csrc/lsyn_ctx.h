@@ -148,7 +148,7 @@ struct lsyn_ctx {
   cudaEvent_t ev_side[2] = {};       // 0: the main stream reached the reset; 1: the big table is clear
   unsigned max_entries = 0;
   DevCounters* ctr = nullptr;
-  uint4* consts = nullptr;  // [5][vecs]: lenmask, label, care, key, mul
+  uint4* consts = nullptr;  // [4][vecs]: lenmask, label, care, mul
   uint4* atoms = nullptr;   // [n_props][vecs]
   unsigned long long* defer[2] = {nullptr, nullptr};
   unsigned defer_cap = 0;
@@ -201,8 +201,7 @@ struct lsyn_ctx {
     cv.lenmask = consts;
     cv.label = consts + vecs;
     cv.care = consts + 2 * vecs;
-    cv.hkey = consts + 3 * vecs;
-    cv.hmul = consts + 4 * vecs;
+    cv.hmul = consts + 3 * vecs;
     cv.atoms = atoms;
     cv.defer_out = defer_out;
     cv.defer_out_n = defer_out_n;

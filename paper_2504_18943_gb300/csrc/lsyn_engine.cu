@@ -287,7 +287,7 @@ lsyn_status Engine::bind(Job* j, int slot) {
   if (!reserve_slot(s, j, &err)) return LSYN_E_CUDA;
   lsyn_ctx* c = j->c;
   const size_t M = size_t(c->vecs) * 16;
-  if (!s.misc.grow(pool_, (5 + size_t(c->n_props)) * M, &err)) return LSYN_E_NOMEM;
+  if (!s.misc.grow(pool_, (4 + size_t(c->n_props)) * M, &err)) return LSYN_E_NOMEM;
   s.job = j;
   s.tcap = 0;
   j->slot = slot;
@@ -296,7 +296,7 @@ lsyn_status Engine::bind(Job* j, int slot) {
   c->slotpos = static_cast<unsigned*>(s.slotpos.ptr());
   c->homes = static_cast<unsigned*>(s.homes.ptr());
   c->consts = static_cast<uint4*>(s.misc.ptr());
-  c->atoms = c->consts + size_t(5) * c->vecs;
+  c->atoms = c->consts + size_t(4) * c->vecs;
   c->defer[0] = static_cast<unsigned long long*>(s.defer[0].ptr());
   c->defer[1] = static_cast<unsigned long long*>(s.defer[1].ptr());
   c->table = static_cast<unsigned long long*>(s.table[s.cur_table].ptr());

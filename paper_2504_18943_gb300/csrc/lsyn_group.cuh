@@ -25,10 +25,10 @@
 // that runs out.
 //
 // Measured against the kernels that walked a matrix with one warp (complete
-// levels, one GB300): 10 propositions, 2048 traces (16 KiB), levels 1-7 in 8.9
+// levels, one GB300): 10 propositions, 2048 traces (16 KiB), levels 1-7 in 8.6
 // ms instead of 12.1; 3 propositions, 250 traces of up to 64 positions (2000
-// bytes), levels 1-10 in 5.0 ms instead of 6.7; 200 traces of up to 200
-// positions (four words each), levels 1-9 in 4.7 ms instead of 13.7. The level
+// bytes), levels 1-10 in 4.2 ms instead of 6.8; 200 traces of up to 200
+// positions (four words each), levels 1-9 in 4.3 ms instead of 13.8. The level
 // kernels of the last levels then run at 3.8-5.0 TB/s of algorithmic bytes (3.0-3.8
 // with four words), bound by instructions and the latency that 24 warps an SM
 // hide; levels below 10^4 candidates take 12-20 us a launch instead of 40-440.

@@ -103,7 +103,6 @@ struct CacheView {
   const uint4* lenmask;          // [vecs]: bits 0..len-1 of every trace word
   const uint4* label;            // [vecs]: bit 0 = 1 for positive traces
   const uint4* care;             // [vecs]: bit 0 = 1 for real (not padding) traces
-  const uint4* hkey;             // [vecs]: per-32-bit-word hash keys
   const uint4* hmul;             // [vecs]: per-32-bit-word odd hash multipliers
   const uint4* atoms;            // [n_props][vecs]
   unsigned long long* defer_out; // deferred descriptors written by this launch
