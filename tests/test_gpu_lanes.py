@@ -87,3 +87,21 @@ def test_large_level_with_little_room_or_log(L):
         with L.Synthesizer(p, config) as s:
             got = [s.level(k) for k in range(1, depth + 1)]
         assert [st.unique for st in got] == sizes and not got[-1].cache_full
+
+
+@pytest.mark.parametrize("traces,bits", [(4, 32), (2, 64), (7, 32), (4, 64), (14, 32), (8, 64), (30, 32), (15, 64)])
+def test_grammars_without_some_operators(L, traces, bits):
+    """The launches with the paper's operators compiled in build the levels of
+    its grammar and of parts of it (a fixed tile gives every level launches of
+    its own)."""
+    p = _problem(2, traces, 5, 30, bits, seed=11)
+    for ops in (L.OPS_PAPER, L.OP_X | L.OP_U, L.OP_NOT | L.OP_AND, L.OPS_PAPER | L.OP_OR, L.OPS_PAPER | L.OP_G):
+        run = oracle.Spec.from_problem(p).enumerate(7, ops)
+        config = L.torch_config(op_mask=ops, cache_bytes=64 << 20, full_levels=True)
+        config.tile_rows = 8
+        with L.Synthesizer(L.pack_problem(p), config) as s:
+            for k in range(1, 8):
+                assert s.level(k).unique == run.size(k), (ops, k)
+                if run.size(k):
+                    want = U.sorted_rows(U.oracle_level_words(run, k, p.traces.lengths, bits))
+                    assert np.array_equal(U.sorted_rows(s.export(k)), want), (ops, k)

@@ -90,3 +90,32 @@ def test_arena_fills_in_a_small_level(L, traces, bits, row):
         assert status == L.LSYN_E_CACHE_FULL and res.levels_done == 5
         assert [lv.unique for lv in levels[:4]] == sizes[:4]
         assert levels[4].cache_full == 1 and levels[4].unique == room - sum(sizes[:4])
+
+
+def test_threads_solve_small_problems_at_once(L):
+    """Eight threads, each with a context and a stream of its own, solve at
+    once: the launches whose blocks wait for one another do not wait for those
+    of another launch, and every solve has the answer it has alone."""
+    import threading
+    import torch
+    packed = [L.pack_problem(W.tiny_problem(s, oracle.labeller)) for s in range(4)]
+    packed += [L.pack_problem(W.batched_problem(1000, i, oracle.labeller)) for i in range(4)]
+
+    def solve(i, out, n):
+        stream = torch.cuda.Stream()
+        with L.Synthesizer(packed[i], L.make_config(cache_bytes=64 << 20, stream=stream.cuda_stream)) as s:
+            for _ in range(n):
+                s.reset()
+                status, res, _, _ = s.solve(7)
+                out[i].add((status, res.size))
+
+    alone = [set() for _ in packed]
+    for i in range(len(packed)):
+        solve(i, alone, 1)
+    out = [set() for _ in packed]
+    threads = [threading.Thread(target=solve, args=(i, out, 100)) for i in range(len(packed))]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert out == alone
