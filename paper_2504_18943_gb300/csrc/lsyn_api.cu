@@ -836,7 +836,7 @@ lsyn_status small_levels(lsyn_ctx* c, int k, int last, lsyn_level_stats* out, in
   if (c->timing) cudaEventRecord(c->ev[0], c->stream);
   e = c->word_bits == 32 ? SmallKernels<uint32_t>::run(cv, c->small_how, a, c->small, c->stream)
                          : SmallKernels<uint64_t>::run(cv, c->small_how, a, c->small, c->stream);
-  if (e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorNotSupported) {
+  if (e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorNotSupported || e == cudaErrorLaunchOutOfResources) {
     cudaGetLastError();  // (not on the devices this is built for) the levels' own launches do
     c->small_off = true;
     return LSYN_OK;

@@ -315,6 +315,26 @@ __global__ void __launch_bounds__(256, 2) k_small_group(CacheView cv, const __gr
 // ---------------------------------------------------------------------------
 // Launcher
 // ---------------------------------------------------------------------------
+// The limit of a kernel's dynamic shared memory belongs to the function, not to
+// a context or a launch: raised once, to all that a block may have beside the
+// kernel's static shared memory. (Set to each context's own need, it went down
+// under the contexts with wider matrices, whose launches were then refused.)
+template <typename W, bool MP>
+cudaError_t small_group_limit() {
+  static const cudaError_t set = [] {
+    const void* fn = (const void*)k_small_group<W, MP>;
+    cudaFuncAttributes fa{};
+    int dev = 0, optin = 0;
+    cudaError_t e = cudaFuncGetAttributes(&fa, fn);
+    if (e == cudaSuccess) e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - int(fa.sharedSizeBytes));
+    return e;
+  }();
+  return set;
+}
+
 template <typename W>
 cudaError_t SmallKernels<W>::prepare(const CacheView& cv, int sms, SmallLaunch* out) {
   const void* fn = nullptr;
@@ -342,7 +362,7 @@ cudaError_t SmallKernels<W>::prepare(const CacheView& cv, int sms, SmallLaunch* 
       blocks_per_sm = unsigned(per_sm);
       if (smem <= 100 * 1024) break;  // two blocks fit an SM
     }
-    const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+    const cudaError_t e = cv.planes > 1 ? small_group_limit<W, true>() : small_group_limit<W, false>();
     if (e != cudaSuccess) return e;
     group_shape(cv, kGroupList, 1, unsigned(sms) * blocks_per_sm * unsigned(kGroupMaxWarps), &g);
     out->list_warps = unsigned(g.warps);
