@@ -359,7 +359,7 @@ void lsyn::ctx_level_plan(lsyn_ctx* c, int k, LevelPlan* lp) {
   //   faster than the counter takes them (one in 1.3 ns): there, up to
   //   kLanesAhead, if every candidate would fit beside all that the warps can
   //   leave over (two launches, up to 64 warps an SM), so that no id left over
-  //   can fill the cache, and if the log takes theirs. 64-byte matrices, whole
+  //   can fill the cache, and if the log and its bitmap take theirs. 64-byte matrices, whole
   //   level, exact against ahead: 137 / 146 us at 0.74 M candidates (no holes to
   //   close), 245 / 235 at 2.5 M, 1590 / 1370 at 28 M;
   // - a few in a large level of path C, where a batch seldom claims fewer: no
@@ -370,8 +370,9 @@ void lsyn::ctx_level_plan(lsyn_ctx* c, int k, LevelPlan* lp) {
     const long long cand = level_candidate_count(c, k);
     c->chunk = 1;
     if (c->path == 1) {
-      const unsigned long long over = (unsigned long long)c->sms * 64ull * 2ull * kLanesAhead;
-      if (cand > (1ll << 20) && (unsigned long long)cand + over <= free_ids && c->hole_cap >= 1u << 16)
+      const unsigned long long over = lanes_left_over(c->sms);
+      if (cand > (1ll << 20) && (unsigned long long)cand + over <= free_ids &&
+          lanes_ranges(c->sms) <= c->hole_cap && over <= 32ull * c->hole_cap)
         c->chunk = kLanesAhead;
     } else if (c->path == 2) {
       const unsigned long long warps = (unsigned long long)c->sms * 24ull;

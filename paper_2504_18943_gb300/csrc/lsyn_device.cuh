@@ -1866,9 +1866,9 @@ __device__ __forceinline__ unsigned block_scan_1024(unsigned v, unsigned* total)
 // dense end is total - H. The entries in [dense_end, total) (ids in no hole,
 // in id order) are the sources and the hole ids below dense_end (in log order)
 // the destinations of the moves, paired by rank: both lists have the same
-// length. Each logged range is at most 32 ids (a warp reserves at most 32 ids
-// at a time), so H <= 32 x hole_cap and the bitmap of [dense_end, total) fits
-// hole_cap words.
+// length. The bitmap of [dense_end, total) takes H / 32 of hole_cap words: a
+// logged range of path C is at most 4 ids, and path A reserves ahead only where
+// all that its warps can leave over (lsyn_ids.h) fits.
 //
 // Scratch layout (3 x hole_cap + 32 words): header [16] = {H, dense_end,
 // words, n}, bits [hole_cap] (holes in [dense_end, total)), word_pref

@@ -6,6 +6,8 @@
 #include <string>
 #include <cuda_runtime.h>
 
+#include "lsyn_ids.h"
+
 namespace lsyn {
 
 // This thread's message for lsyn_last_error(NULL).
@@ -47,8 +49,6 @@ constexpr uint32_t kSlotTomb = 0xFFFFFFFEu;     // claimed, but the arena was fu
 // the batch kernels).
 constexpr int kLaunchKinds = 4;
 constexpr unsigned kKindUnary = 0, kKindBinary = 1, kKindOther = 2;
-// Ids that a warp of a large path-A level reserves beyond its need.
-constexpr unsigned kLanesAhead = 64;
 
 struct alignas(128) DevCounters {
   // ---- the id counter (an atomic per warp batch with claims) ----

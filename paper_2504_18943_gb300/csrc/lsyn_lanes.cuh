@@ -85,11 +85,11 @@ __device__ __forceinline__ void lanes_run(const CacheView& cv, const LanesWork& 
 #pragma unroll
   for (int r = 0; r < R; ++r) pend_pos[r] = pend_tag[r] = pend_id[r] = 0;
   unsigned built = 0, inserted = 0, iter = 0;  // (a warp's share of a level fits 32 bits)
-  unsigned ids_next = 0, ids_end = 0;  // ids reserved and not used yet
+  IdStock ids;
   // All warps' reservations meet at one counter. In a large level a warp
-  // reserves up to kLanesAhead ids more than the empty slots it has just met, in
-  // the same atomic, beside the claims themselves; fewer towards its last batch,
-  // so that almost none are left over (holes, to be closed).
+  // reserves up to kLanesAhead ids more than its claims need, in the same
+  // atomic; fewer towards its last batch, so that almost none are left over
+  // (holes, to be closed).
   const bool ahead = cv.chunk > 1u && !lw.exact;
   unsigned batches = total > warp * NG ? unsigned((total - warp * NG - 1) / (nwarps * NG)) : 0u;  // after this one
   bool full = false;  // the arena is full: the specification check only
@@ -243,7 +243,7 @@ __device__ __forceinline__ void lanes_run(const CacheView& cv, const LanesWork& 
       // reads its bucket again in the next round.
       uint32_t cmp[R], claim[R];
       int won[R];  // the claim's outcome
-      unsigned n_empty = 0, n_claim = 0, asked = 0, fresh = 0;
+      unsigned n_claim = 0;
 #pragma unroll
       for (int r = 0; r < R; ++r) {
         cmp[r] = 0u;  // id + 1 of the row to compare with
@@ -263,11 +263,6 @@ __device__ __forceinline__ void lanes_run(const CacheView& cv, const LanesWork& 
           }
         }
         if (empty) won[r] = claim_slot(cv.table + pos[r], tag[r]);
-        n_empty += unsigned(__popc(__ballot_sync(kFull, empty)));
-      }
-      if (ahead && n_empty > ids_end - ids_next) {
-        asked = n_empty - (ids_end - ids_next) + min(kLanesAhead, 2u * batches);
-        if (lane == 0) fresh = atomicAdd(&cv.ctr->n_entries, asked);
       }
       __syncwarp();  // the probing lanes' acquires, before every lane's row reads
       uint4 st[NO];
@@ -298,19 +293,19 @@ __device__ __forceinline__ void lanes_run(const CacheView& cv, const LanesWork& 
         n_claim += unsigned(__popc(claim[r]));
       }
       // claims: ids (the warp's stock, then the fresh ones), rows written by the groups
-      if (n_claim | asked) {
-        const unsigned have = ids_end - ids_next;
-        if (asked == 0u && n_claim > have) {
-          asked = n_claim - have;
+      if (n_claim) {
+        const unsigned asked = ids.ask(n_claim, ahead ? min(kLanesAhead, 2u * batches) : 0u);
+        unsigned fresh = 0;
+        if (asked) {
           if (lane == 0) fresh = atomicAdd(&cv.ctr->n_entries, asked);
+          fresh = __shfl_sync(kFull, fresh, 0);
         }
-        if (asked) fresh = __shfl_sync(kFull, fresh, 0);
         uint32_t id1[R];  // id + 1 of a row to write
         unsigned rank0 = 0;
 #pragma unroll
         for (int r = 0; r < R; ++r) {
           const unsigned rank = rank0 + unsigned(__popc(claim[r] & ((1u << lane) - 1u)));
-          const unsigned id = rank < have ? ids_next + rank : fresh + (rank - have);
+          const unsigned id = ids.id(rank, fresh);
           rank0 += unsigned(__popc(claim[r]));
           const bool ok = state[r] == kClaimed && id < cv.max_entries;
           id1[r] = ok ? id + 1u : 0u;
@@ -338,13 +333,7 @@ __device__ __forceinline__ void lanes_run(const CacheView& cv, const LanesWork& 
           const uint32_t id = from_owner(id1[NO == 4 && V < 4 ? o % R : 0], o);
           if (id) cv.arena[size_t(id - 1u) * V + l] = c[o];
         }
-        if (n_claim >= have) {
-          ids_next = asked ? fresh + (n_claim - have) : ids_end;
-          ids_end = asked ? fresh + asked : ids_end;
-        } else {
-          ids_next += n_claim;
-          if (asked && lane == 0) WarpDedup::log_hole(cv, fresh, fresh + asked);  // (rare: most claims were lost)
-        }
+        ids.use(n_claim, asked, fresh);
       }
       bool more = false;
 #pragma unroll
@@ -405,7 +394,7 @@ __device__ __forceinline__ void lanes_run(const CacheView& cv, const LanesWork& 
   }
   flush();
   if (lane == 0) {
-    WarpDedup::log_hole(cv, ids_next, ids_end);
+    WarpDedup::log_hole(cv, ids.next, ids.end);
     if (inserted) atomicAdd(&cv.ctr->inserted_k[kKind], (unsigned long long)inserted);
     if (MODE != kLanesList && built) atomicAdd(&cv.ctr->built_k[kKind], (unsigned long long)built);
     if (MODE == kLanesList && lw.atoms && blockIdx.x == 0 && threadIdx.x == 0)

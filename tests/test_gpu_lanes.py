@@ -105,3 +105,16 @@ def test_grammars_without_some_operators(L, traces, bits):
                 if run.size(k):
                     want = U.sorted_rows(U.oracle_level_words(run, k, p.traces.lengths, bits))
                     assert np.array_equal(U.sorted_rows(s.export(k)), want), (ops, k)
+
+
+def test_level_of_half_a_billion_candidates(L):
+    """32-byte matrices: a level of 5 x 10^8 candidates, whose warps reserve ids
+    ahead and lose claims to one another in every few batches, is complete and
+    the same as without any reserved ahead (a hole log that is too small)."""
+    p = L.pack_problem(_problem(2, 8, 8, 32, 32, seed=5))
+    got = []
+    for hole_cap in (0, 1):
+        with L.Synthesizer(p, L.make_config(cache_bytes=40 << 30, full_levels=True, hole_cap=hole_cap)) as s:
+            got.append([(st.candidates, st.unique, st.cache_full) for st in (s.level(k) for k in range(1, 16))])
+    assert got[0] == got[1]
+    assert got[0][-1][0] > 4 * 10 ** 8 and not got[0][-1][2]
