@@ -47,6 +47,12 @@ constexpr int kGroupMaxWarps = 8;  // warps that share a candidate (a block)
 // 5-7 %.
 constexpr int kGroupVecs = 16;
 constexpr int kGroupMaxBatch = 4;  // left rows per item
+// A group hands its count of candidates in when it gets here: a level may have
+// more of them than 32 bits hold for each group, above all one that goes on with
+// the specification check alone in a full arena. The check costs 0.4 % of the
+// kernels of 2 and 16 KiB matrices; a 64-bit count 1 %, as a register or in
+// shared memory, a count in every lane 1.7 %, the check at the item's end 4 %.
+constexpr unsigned kCountMost = 1u << 31;
 constexpr unsigned kGroupWaits = 12;   // probes of a pending slot (a round trip and two barriers each) before deferring
 
 // Blocks per SM that the compiler is to leave registers for: three (80
@@ -338,7 +344,7 @@ __device__ __forceinline__ void group_run(const CacheView& cv, const GroupWork& 
   constexpr int kProbing = WarpDedup::kProbing, kDone = WarpDedup::kDone, kClaimed = WarpDedup::kClaimed;
   constexpr int kCompare = 4, kWait = 5, kTwin = 6;
   WarpDedup::Pending pend;
-  unsigned built = 0, inserted = 0;  // (a warp's share of a level fits 32 bits)
+  unsigned built = 0, inserted = 0;  // (ids fit 32 bits; candidates: see kCountMost)
 
   while (true) {
     const int n = int(uniform(ctl->n[cur]));
@@ -431,6 +437,10 @@ __device__ __forceinline__ void group_run(const CacheView& cv, const GroupWork& 
       }
       WarpDedup::flush(pend);  // the previous item's rows: the group never meets its own claims as pending
       built += __popc(mine_m);
+      if (built >= kCountMost) {
+        if (MODE != kGroupList && lane == 0) atomicAdd(&cv.ctr->built_k[kKind], (unsigned long long)built);
+        built = 0;
+      }
     }
 
     bool first = true;

@@ -84,14 +84,17 @@ __device__ __forceinline__ void lanes_run(const CacheView& cv, const LanesWork& 
   uint32_t pend_pos[R], pend_tag[R], pend_id[R];  // claimed slots whose rows are written: id + 1, 0 = none
 #pragma unroll
   for (int r = 0; r < R; ++r) pend_pos[r] = pend_tag[r] = pend_id[r] = 0;
-  unsigned built = 0, inserted = 0, iter = 0;  // (a warp's share of a level fits 32 bits)
+  unsigned long long built = 0;
+  static_assert(sizeof(built) == sizeof(cv.ctr->built_k[0]), "a warp's share of a level may need all of its bits");
+  unsigned inserted = 0, iter = 0;  // (ids fit 32 bits)
   IdStock ids;
   // All warps' reservations meet at one counter. In a large level a warp
   // reserves up to kLanesAhead ids more than its claims need, in the same
   // atomic; fewer towards its last batch, so that almost none are left over
   // (holes, to be closed).
   const bool ahead = cv.chunk > 1u && !lw.exact;
-  unsigned batches = total > warp * NG ? unsigned((total - warp * NG - 1) / (nwarps * NG)) : 0u;  // after this one
+  // batches after this one (with `ahead`, the level's candidates fit 32 bits)
+  unsigned batches = total > warp * NG ? unsigned((total - warp * NG - 1) / (nwarps * NG)) : 0u;
   bool full = false;  // the arena is full: the specification check only
 
   // As WarpDedup::flush: the warp barrier orders the other lanes' row stores
@@ -396,7 +399,7 @@ __device__ __forceinline__ void lanes_run(const CacheView& cv, const LanesWork& 
   if (lane == 0) {
     WarpDedup::log_hole(cv, ids.next, ids.end);
     if (inserted) atomicAdd(&cv.ctr->inserted_k[kKind], (unsigned long long)inserted);
-    if (MODE != kLanesList && built) atomicAdd(&cv.ctr->built_k[kKind], (unsigned long long)built);
+    if (MODE != kLanesList && built) atomicAdd(&cv.ctr->built_k[kKind], built);
     if (MODE == kLanesList && lw.atoms && blockIdx.x == 0 && threadIdx.x == 0)
       atomicAdd(&cv.ctr->built_k[kKind], total);  // deferred candidates were counted when first built
   }
