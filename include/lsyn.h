@@ -173,7 +173,15 @@ typedef struct {
   double time_limit_ms;
 } lsyn_config;
 
-/* Per-level statistics (filled by lsyn_enumerate_level). */
+/*
+ * Per-level statistics (filled by lsyn_enumerate_level and lsyn_solve). A small
+ * level (up to some 10^5 candidates, without time_limit_ms and tile_rows) is
+ * built by one launch for both kinds of operators and, in lsyn_solve, for
+ * several levels: its device time is kernel_ms[3] ("other"), with nothing in
+ * the unary, binary and resolve fields; the launch and what the call took
+ * beside the device's time count for the first of its levels, so that sums over
+ * levels are those of the call. bytes_unary and bytes_binary keep to the operators.
+ */
 typedef struct {
   int32_t level;          /* k */
   int32_t solved;         /* 1 if a candidate of this level separates (P, N) */
@@ -183,12 +191,13 @@ typedef struct {
   int64_t unique;         /* new characteristic matrices added to the cache: |L_k| */
   int64_t total;          /* entries in the cache after this level */
   int64_t deferred;       /* candidates re-examined after meeting an unpublished slot */
-  double ms;              /* wall time of the level (host clock, includes the final sync) */
+  double ms;              /* wall time of the level (host clock, includes the final sync; of a later
+                             level of a combined launch its time on the device) */
   double kernel_ms[4];    /* with timing=1: device time of the unary, binary, resolve and other launches */
   double bytes_alg;       /* algorithmic bytes of the level (operand reads, probes, compares, inserts) */
-  double bytes_binary;    /* the part of bytes_alg moved by the binary-operator launch */
-  double bytes_unary;     /* the part of bytes_alg moved by the unary-operator launch */
-  int32_t launches;       /* kernel launches issued for this level */
+  double bytes_binary;    /* the part of bytes_alg moved by the binary operators' candidates */
+  double bytes_unary;     /* the part of bytes_alg moved by the unary operators' candidates */
+  int32_t launches;       /* kernel launches issued for this level (0: built by an earlier level's) */
   int32_t reserved;
 } lsyn_level_stats;
 

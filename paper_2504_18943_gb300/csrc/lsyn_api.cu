@@ -891,6 +891,7 @@ lsyn_status small_levels(lsyn_ctx* c, int k, int last, lsyn_level_stats* out, in
     if (st != LSYN_OK) return st;
     level_bytes(c, kk, h, lp, &out[i]);
     out[i].ms = double(r.ns) * 1e-6;
+    if (c->timing) out[i].kernel_ms[3] = out[i].ms;
     if (i) others += out[i].ms;
     ++*built;
   }
@@ -898,7 +899,8 @@ lsyn_status small_levels(lsyn_ctx* c, int k, int last, lsyn_level_stats* out, in
     out[0].launches = 1;
     out[0].ms = std::max(out[0].ms, lsyn::now_ms() - t0 - others);
     float ms = 0;
-    if (c->timing && cudaEventElapsedTime(&ms, c->ev[0], c->ev[1]) == cudaSuccess) out[0].kernel_ms[3] = ms;
+    if (c->timing && cudaEventElapsedTime(&ms, c->ev[0], c->ev[1]) == cudaSuccess)
+      out[0].kernel_ms[3] = std::max(out[0].kernel_ms[3], double(ms) - others);
   }
   return LSYN_OK;
 }

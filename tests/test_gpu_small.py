@@ -119,3 +119,20 @@ def test_threads_solve_small_problems_at_once(L):
     for t in threads:
         t.join()
     assert out == alone
+
+
+@pytest.mark.parametrize("shape", [(3, 31, 8, 32, 32, 6), (2, 200, 8, 60, 64, 5)])
+def test_timed_levels_have_their_time_and_launches(L, shape):
+    """With timing on, every level of a solve has device time, whichever launch
+    built it, and the levels' times and launches add up to the call's."""
+    props, traces, lo, hi, bits, depth = shape
+    packed = L.pack_problem(_noise(props, traces, lo, hi, bits))
+    with L.Synthesizer(packed, L.make_config(cache_bytes=256 << 20, timing=True)) as s:
+        s.solve(depth)
+        s.reset()
+        status, res, _, levels = s.solve(depth)
+        assert status == L.LSYN_NOT_FOUND and len(levels) == depth
+        for lv in levels:
+            assert 0 < sum(lv.kernel_ms) and 0 < lv.ms
+        assert sum(sum(lv.kernel_ms) for lv in levels) <= sum(lv.ms for lv in levels) <= res.ms
+        assert sum(lv.launches for lv in levels) == res.launches >= 1
