@@ -665,10 +665,16 @@ def run_served(args):
     return 0
 
 
+def _kernel_sources():
+    """The files that the level kernels and their launches are compiled from."""
+    csrc = os.path.join(ROOT, "paper_2504_18943_gb300", "csrc")
+    return sorted(n for n in os.listdir(csrc) if n.endswith(".cuh")) + ["lsyn_api.cu", "lsyn_internal.h", "lsyn_ids.h"]
+
+
 def _kernel_sha() -> str:
     import hashlib
     h = hashlib.sha256()
-    for name in ("lsyn_device.cuh", "lsyn_group.cuh", "lsyn_lanes.cuh", "lsyn_api.cu", "lsyn_internal.h"):
+    for name in _kernel_sources():
         with open(os.path.join(ROOT, "paper_2504_18943_gb300", "csrc", name), "rb") as f:
             h.update(f.read())
     return h.hexdigest()[:16]
