@@ -826,7 +826,6 @@ lsyn_status small_levels(lsyn_ctx* c, int k, int last, lsyn_level_stats* out, in
     a.level_start[i] = c->level_start[size_t(i)];
     a.level_n[i] = c->level_n[size_t(i)];
   }
-  const LaunchCfg lc{c->stream, c->sms};
   c->level_budget_ns = 0;
   const CacheView cv = c->view(c->defer[0], &c->ctr->defer_n[0]);
   cudaError_t e = cudaSuccess;
@@ -875,19 +874,8 @@ lsyn_status small_levels(lsyn_ctx* c, int k, int last, lsyn_level_stats* out, in
     h.sol = r.sol;
     h.solved = r.solved;
     h.full = r.full;
-    uint32_t total = r.total;
-    if (r.holes) {  // (rare) the last level of the launch: close them as any level's
-      e = c->word_bits == 32
-              ? Kernels<uint32_t>::close_holes(cv, lp.start, c->hole_bits, c->moves, c->move_cap, lc)
-              : Kernels<uint64_t>::close_holes(cv, lp.start, c->hole_bits, c->moves, c->move_cap, lc);
-      if (e == cudaSuccess)
-        e = cudaMemcpyAsync(&c->h_snap[0].c, c->ctr, sizeof(DevCounters), cudaMemcpyDeviceToHost, c->stream);
-      if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
-      if (e != cudaSuccess) return c->cuda_fail(e, "hole fixup kernels");
-      if (c->h_snap[0].c.error) return check_failed(c, c->h_snap[0].c.error);
-      total = std::min(c->h_snap[0].c.n_entries, c->max_entries);
-    }
-    const lsyn_status st = lsyn::ctx_commit_level(c, kk, h, total, r.deferred, lp, &out[i]);
+    if (r.holes) return check_failed(c, 4);  // ids are reserved exactly: nothing logs any
+    const lsyn_status st = lsyn::ctx_commit_level(c, kk, h, r.total, r.deferred, lp, &out[i]);
     if (st != LSYN_OK) return st;
     level_bytes(c, kk, h, lp, &out[i]);
     out[i].ms = double(r.ns) * 1e-6;

@@ -475,15 +475,6 @@ struct PathA {
     uint4 lm[V], lab[V], care[V], mul[V];
   };
 
-  __device__ static void load_consts(const CacheView& cv, Consts* s) {
-    for (int i = threadIdx.x; i < V; i += blockDim.x) {
-      s->lm[i] = cv.lenmask[i];
-      s->lab[i] = cv.label[i];
-      s->care[i] = cv.care[i];
-      s->mul[i] = cv.hmul[i];
-    }
-  }
-
   __device__ static void load_row(const uint4* p, uint4 (&x)[V]) {
 #pragma unroll
     for (int v = 0; v < V; ++v) x[v] = __ldg(p + v);
@@ -545,14 +536,6 @@ struct PathA {
     }
     atomicExch(&cv.ctr->error, 1u);
     return 0;
-  }
-
-  __device__ static unsigned candidate(const CacheView& cv, const Consts& s, uint32_t op, const uint4 (&a)[V],
-                                       const uint4 (&b)[V], uint64_t desc, bool full) {
-    uint4 c[V];
-#pragma unroll
-    for (int v = 0; v < V; ++v) c[v] = v_op<W>(op, a[v], b[v], s.lm[v], cv.steps);
-    return process(cv, s, c, desc, full);
   }
 };
 
