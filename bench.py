@@ -36,6 +36,7 @@ WORKLOAD = "mid-scale plain solve: 5 props, 64+64 traces, len U[8,32], Bernoulli
 METRIC = "unique formulas/sec"
 CACHE_BYTES = 64 << 30
 MAX_SIZE = 16
+FORMULA_READ_BYTES = 1024 + 4  # a formula's text and its status, as lsyn_solve reads them from the device
 LARGE_CACHE_BYTES = 150 * 10**9
 LARGE_WORKLOAD = ("large plain solve: 10 props, 1024+1024 traces, len U[16,64], Bernoulli(p) with p U[0.2,0.8] per "
                   "prop, hidden size 15, 2048 x uint64 words (16 KiB) per CM, 150 GB cache; every level built "
@@ -391,7 +392,7 @@ def run_lsyn(args):
                                        "ms": kms[n]} for n in kms if n != dom}},
             "cpu_baseline": cpu,
             "e2e": {"value": e2e_total / (e2e_ms / 1000.0) if e2e_ms > 0 else None, "unit": "unique formulas/sec",
-                    "h2d_bytes_per_step": packed.h2d_bytes, "d2h_bytes_per_step": 1 << 16,
+                    "h2d_bytes_per_step": packed.h2d_bytes, "d2h_bytes_per_step": FORMULA_READ_BYTES,
                     "steps": e2e_steps, "l2_flush": True},
             "gpu_launches": launches,
             "clocks": clocks.summary(),

@@ -1,5 +1,6 @@
-"""The bench's traffic record holds for the sources it was taken from: the hash
-that says so covers every file that the kernels' translation units include."""
+"""What the bench states about the sources: the hash that ties the traffic record
+to the kernels covers every file that their translation units include, and the
+bytes read back for a formula are those that the library copies."""
 from __future__ import annotations
 
 import glob
@@ -18,6 +19,14 @@ def _included(name, seen):
                 seen.add(inc)
                 _included(inc, seen)
     return seen
+
+
+def test_formula_read_is_counted_as_it_is_made():
+    """The end-to-end line's device-to-host bytes are those that the library
+    copies for a formula of ordinary length."""
+    with open(os.path.join(CSRC, "lsyn_api.cu")) as f:
+        got = int(re.search(r"size_t got = (\d+);", f.read()).group(1))
+    assert bench.FORMULA_READ_BYTES == got + 4
 
 
 def test_traffic_record_covers_the_kernels_sources():
