@@ -360,8 +360,8 @@ void lsyn::ctx_level_plan(lsyn_ctx* c, int k, LevelPlan* lp) {
   //   kLanesAhead, if every candidate would fit beside all that the warps can
   //   leave over (two launches, up to 64 warps an SM), so that no id left over
   //   can fill the cache, and if the log and its bitmap take theirs. 64-byte matrices, whole
-  //   level, exact against ahead: 137 / 146 us at 0.74 M candidates (no holes to
-  //   close), 245 / 235 at 2.5 M, 1590 / 1370 at 28 M;
+  //   level, exact against ahead: 203 / 192 us at 2.5 M candidates, 534 / 455 at
+  //   8.5 M, 1518 / 1307 at 28 M, 4812 / 4094 at 92 M;
   // - a few in a large level of path C, where a batch seldom claims fewer: no
   //   faster than none (6.92 ms at 52 M candidates; 7.12 with 32 at a time), no
   //   slower but for the close (6 us), and the hole log keeps its use.

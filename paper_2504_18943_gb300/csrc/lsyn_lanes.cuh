@@ -19,8 +19,10 @@
 // Measured against one thread per CM (complete levels, one GB300): 30 traces
 // (120 bytes), four propositions, levels 1-10 in 2.6 ms instead of 5.2, the
 // last level's binary launch 13.2 G candidates/s instead of 4.8; 14 traces (56
-// bytes), the paper's grammar, levels 1-15 in 7.9 ms instead of 8.5: up to 2.5x
-// faster on launches of 10^5 to 10^7 candidates, 21.5 G/s at 28 M.
+// bytes), the paper's grammar, levels 1-15 in 8.2 ms instead of 8.9: up to 2.5x
+// faster on launches of 10^5 to 10^7 candidates, 22.3 G/s at 28 M. (A loop with
+// the same accesses and nothing else - a random bucket a candidate, a random
+// 64-byte row of 4 GiB for 27 of 32, a claim and a row written for 5 - does 20 G/s.)
 #pragma once
 
 #include "lsyn_device.cuh"
@@ -50,7 +52,9 @@ struct LanesWork {
 // those of the paper's grammar (not, X, F; and, U), whose launches then hash,
 // compare and write a quarter less. 64-byte matrices, 92 M candidates of that
 // grammar: 886 + 3690 us (unary + binary) with all four compiled in, 859 + 3455
-// with three. Two operators compiled in were not tried: no grammar here has them.
+// with three (now 919 + 3932 with ids exactly as claimed, 876 + 3184 with ids
+// ahead, see ctx_level_plan). Two operators compiled in were not tried: no grammar
+// here has them.
 template <typename W, int V, int MODE, bool kFresh, unsigned kOps>
 __device__ __forceinline__ void lanes_run(const CacheView& cv, const LanesWork& lw, const BinaryPlan& plan) {
   constexpr unsigned kKind = MODE == kLanesUnary ? kKindUnary : MODE == kLanesBinary ? kKindBinary : kKindOther;

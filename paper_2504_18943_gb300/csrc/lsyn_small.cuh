@@ -20,9 +20,9 @@
 //
 // Measured (one GB300): a level of 10^1 to 10^4 candidates in 10-15 us inside a
 // solve, 28-45 us as a call of its own, against 55-110 us (up to 1 ms on wide
-// matrices, before the group kernels); a tiny problem's reset and solve 165 us
-// instead of 319 (of which about 100 are the caller's Python), levels 1-10 of 250
-// traces 4.44 ms instead of 4.66. Two blocks per SM (up to 128 registers, three
+// matrices, before the group kernels); a tiny problem's reset and solve 135 us
+// instead of 170 or 168 instead of 319, by the problem (about 100 are the
+// caller's Python), levels 1-10 of 250 traces 4.44 ms instead of 4.66. Two blocks per SM (up to 128 registers, three
 // kinds of step in one kernel): beyond kSmallCandidates a level's own launches
 // are faster.
 #pragma once
